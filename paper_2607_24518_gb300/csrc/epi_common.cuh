@@ -135,6 +135,125 @@ __device__ __forceinline__ void ff_xor_add(float &hi, float &lo, int o) {
   lo = __fsub_rn(t, __fsub_rn(hi, s));
 }
 
+// Running sum of squares as a float-float pair: the product is split exactly
+// by an FMA and the high parts are added by Knuth's TwoSum, so only the low
+// part (near 2^-23 of the sum) is rounded.  FP64 runs at two operations per
+// SM and cycle on this part; a run of 64 entries summed this way (rounding
+// near 2^-47) takes three FP64 operations instead of 128 and more.
+struct SqRun {
+  float h = 0.f, l = 0.f, m = 0.f;  // sum = h + l, m = largest magnitude
+  // SHORT: v has at most 12 significant bits, so its square is exact
+  template <bool SHORT = false>
+  __device__ __forceinline__ void add(float v) {
+    const float p = __fmul_rn(v, v);
+    const float t = __fadd_rn(h, p), b = __fsub_rn(t, h);
+    float e = __fadd_rn(__fsub_rn(h, __fsub_rn(t, b)), __fsub_rn(p, b));
+    if constexpr (!SHORT) e = __fadd_rn(e, fmaf(v, v, -p));
+    l = __fadd_rn(l, e);
+    h = t;
+    m = fmaxf(m, fabsf(v));
+  }
+  // squares that neither overflow nor lose bits to underflow; otherwise the
+  // caller sums the run in FP64
+  __device__ __forceinline__ bool in_range() const {
+    return m < 0x1p56f && (m == 0.f || m > 0x1p-40f);
+  }
+  __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+};
+
+// entry i of S (FP8: the code's value, without its tile scale)
+template <int DT>
+__device__ __forceinline__ float s_entry(const void *S, int64_t i) {
+  if constexpr (DT == 0) return __ldg(reinterpret_cast<const float *>(S) + i);
+  else if constexpr (DT == 1) return bf16_val(__ldg(reinterpret_cast<const uint16_t *>(S) + i));
+  else return e4m3_val(__ldg(reinterpret_cast<const uint8_t *>(S) + i));
+}
+// a lane's 16 entries of columns c0 .. c0 + 511 of a row of S, in 16-byte
+// groups one warp apart (vec: every row starts on a 16-byte boundary), else
+// element by element; entries from column n on are 0.  FP8: the 16 entries
+// are consecutive, so they share a tile scale.
+template <int DT>
+__device__ __forceinline__ void load16(const void *S, int64_t rowbase, int64_t c0, int64_t n,
+                                       bool vec, int lane, float (&v)[16]) {
+  constexpr int W = DT == 0 ? 4 : DT == 1 ? 8 : 16;  // entries of a 16-byte group
+#pragma unroll
+  for (int i = 0; i < 16 / W; ++i) {
+    const int64_t c = c0 + (i * 32 + lane) * W;
+    if (vec && c + W <= n) {
+      const uint4 x = __ldg(reinterpret_cast<const uint4 *>(
+          reinterpret_cast<const uint8_t *>(S) + (rowbase + c) * (16 / W)));
+      const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if constexpr (DT == 0) {
+          v[4 * i + j] = __uint_as_float(w[j]);
+        } else if constexpr (DT == 1) {
+          v[8 * i + 2 * j] = __uint_as_float(w[j] << 16);
+          v[8 * i + 2 * j + 1] = __uint_as_float(w[j] & 0xFFFF0000u);
+        } else {
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const float2 f = __half22float2(__half2(__nv_cvt_fp8x2_to_halfraw2(
+                (__nv_fp8x2_storage_t)(w[j] >> (16 * u)), __NV_E4M3)));
+            v[4 * j + 2 * u] = f.x;
+            v[4 * j + 2 * u + 1] = f.y;
+          }
+        }
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < W; ++j) v[i * W + j] = c + j < n ? s_entry<DT>(S, rowbase + c + j) : 0.f;
+    }
+  }
+}
+
+// the lane's entries of columns [c0, c1) (as load16 deals them) summed in FP64
+template <int DT>
+__device__ __noinline__ double row_sumsq_lane64(const void *S, int64_t rowbase, int64_t c0,
+                                                int64_t c1, int64_t n, const float *scales,
+                                                int lane) {
+  constexpr int W = DT == 0 ? 4 : DT == 1 ? 8 : 16;
+  double acc = 0.0;
+  for (int64_t c = c0 + lane * W; c < c1; c += 32 * W)
+    for (int j = 0; j < W && c + j < n; ++j) {
+      double x = (double)s_entry<DT>(S, rowbase + c + j);
+      if constexpr (DT == 2) x *= (double)scales[(c + j) / kTileRows];
+      acc = fma(x, x, acc);
+    }
+  return acc;
+}
+
+// One lane's share of sum_j S_rj^2 over row r: runs of 64 entries in
+// float-float form, the runs in FP64.  FP8: a power-of-two tile scale (all
+// that symnmf_quantize_fp8 writes) is exact in FP32; other scales and values
+// out of SqRun's range take the FP64 sum.  `scales`: the row's tile scales.
+template <int DT>
+__device__ __forceinline__ double row_sumsq_lane(const void *S, int64_t rowbase, int64_t n,
+                                                 const float *scales, bool vec, int lane) {
+  double acc = 0.0;
+  for (int64_t c0 = 0; c0 < n; c0 += 2048) {
+    SqRun s;
+    bool exact = true;
+    // loads in flight per lane: one chunk of FP32 is four, of FP8 one
+#pragma unroll (DT == 0 ? 1 : DT == 1 ? 2 : 4)
+    for (int i = 0; i < 4; ++i) {
+      const int64_t cc = c0 + 512 * i;
+      if (DT != 2 && cc >= n) break;
+      float v[16], sc = 1.f;
+      load16<DT>(S, rowbase, cc, n, vec, lane, v);
+      if constexpr (DT == 2) {
+        sc = __ldg(scales + min(cc + 16 * lane, n - 1) / kTileRows);
+        exact = exact && (__float_as_uint(sc) & 0x7FFFFFu) == 0u;
+      }
+#pragma unroll
+      for (int j = 0; j < 16; ++j) s.template add<(DT == 2)>(DT == 2 ? v[j] * sc : v[j]);
+    }
+    if (exact && s.in_range()) acc += s.value();
+    else acc += row_sumsq_lane64<DT>(S, rowbase, c0, min(c0 + 2048, n), n, scales, lane);
+  }
+  return acc;
+}
+
 // Sum, in index order, `count` (<= 32) values at base[i * stride]; every
 // load is issued before the ordered additions.
 template <typename T>

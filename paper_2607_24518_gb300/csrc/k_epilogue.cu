@@ -401,42 +401,35 @@ __global__ void __launch_bounds__(256) gram_subset_kernel(const float *gram_part
   o[e] = (float)s;
 }
 
+// ||S||_F^2: one warp per row, runs of 64 entries as float-float sums, runs
+// and rows in FP64.  Bound by HBM; a conversion and a multiply-add per entry
+// in FP64 bounded it by the FP64 pipe before (n=12000 FP8: 1072 -> 74 us,
+// 1.9 TB/s).
 template <int DT>
-__device__ __forceinline__ double s_value(const void *S, int64_t idx, double scale) {
-  if constexpr (DT == 0) {
-    return (double)reinterpret_cast<const float *>(S)[idx];
-  } else if constexpr (DT == 1) {
-    return (double)__bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(S)[idx]);
-  } else {
-    __nv_fp8_e4m3 q;
-    q.__x = reinterpret_cast<const __nv_fp8_storage_t *>(S)[idx];
-    return (double)static_cast<float>(q) * scale;
-  }
-}
-
-template <int DT>
-__global__ void __launch_bounds__(256) norm_s2_kernel(const void *S, int64_t n, int64_t lds,
+__global__ void __launch_bounds__(256, 4) norm_s2_kernel(const void *S, int64_t n, int64_t lds,
                                                       const float *scales, int64_t ld_scales,
-                                                      double *partials) {
+                                                      bool vec, double *partials) {
   __shared__ double red[40];
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * 8;
   double acc = 0.0;
-  for (int64_t r = blockIdx.x; r < n; r += gridDim.x) {
-    for (int64_t c = threadIdx.x; c < n; c += blockDim.x) {
-      const double sc = (DT == 2) ? (double)scales[(r / kTileRows) * ld_scales + c / kTileRows] : 1.0;
-      const double v = s_value<DT>(S, r * lds + c, sc);
-      acc += v * v;
-    }
-  }
+  for (int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); r < n; r += warps)
+    acc += row_sumsq_lane<DT>(S, r * lds, n, scales + (r / kTileRows) * ld_scales, vec, lane);
   acc = block_sum(acc, red);
   if (threadIdx.x == 0) partials[blockIdx.x] = acc;
 }
 
-__global__ void sum_array_kernel(const double *x, int m, int stride, int off, double *out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < m; ++i) s += x[(int64_t)i * stride + off];
-    *out = s;
-  }
+// fixed-order sum of m values: contiguous runs per thread, then the block's
+// order (one thread adding them all took 31 us for 608 values)
+__global__ void __launch_bounds__(256) sum_array_kernel(const double *x, int m, int stride, int off,
+                                                        double *out) {
+  __shared__ double red[40];
+  const int per = (m + 255) / 256;
+  double s = 0.0;
+  for (int i = threadIdx.x * per; i < m && i < (int)(threadIdx.x + 1) * per; ++i)
+    s += x[(int64_t)i * stride + off];
+  s = block_sum(s, red);
+  if (threadIdx.x == 0) *out = s;
 }
 
 // caller row-major n x k -> n x kp over all tile rows (pads zeroed)
@@ -646,13 +639,14 @@ cudaError_t launch_gram_subset(const float *gram_part, int kp, const int *l1, in
 cudaError_t launch_norm_s2(const void *S, int64_t n, int64_t lds, int dtype, const float *scales,
                            int64_t ld_scales, double *partials, int nparts, double *out,
                            cudaStream_t s) {
+  const bool vec = rows_on_16(S, lds, dtype);
   switch (dtype) {
-    case 0: norm_s2_kernel<0><<<nparts, 256, 0, s>>>(S, n, lds, scales, ld_scales, partials); break;
-    case 1: norm_s2_kernel<1><<<nparts, 256, 0, s>>>(S, n, lds, scales, ld_scales, partials); break;
-    case 2: norm_s2_kernel<2><<<nparts, 256, 0, s>>>(S, n, lds, scales, ld_scales, partials); break;
+    case 0: norm_s2_kernel<0><<<nparts, 256, 0, s>>>(S, n, lds, scales, ld_scales, vec, partials); break;
+    case 1: norm_s2_kernel<1><<<nparts, 256, 0, s>>>(S, n, lds, scales, ld_scales, vec, partials); break;
+    case 2: norm_s2_kernel<2><<<nparts, 256, 0, s>>>(S, n, lds, scales, ld_scales, vec, partials); break;
     default: return cudaErrorInvalidValue;
   }
-  sum_array_kernel<<<1, 32, 0, s>>>(partials, nparts, 1, 0, out);
+  sum_array_kernel<<<1, 256, 0, s>>>(partials, nparts, 1, 0, out);
   return cudaGetLastError();
 }
 
@@ -692,7 +686,7 @@ cudaError_t launch_reset(float *A, const float *g, const float *med, float c, in
 
 cudaError_t launch_sum_slot(const double *slots, int ntiles, int which, double *out,
                             cudaStream_t s) {
-  sum_array_kernel<<<1, 32, 0, s>>>(slots, ntiles, kSlotStride, which, out);
+  sum_array_kernel<<<1, 256, 0, s>>>(slots, ntiles, kSlotStride, which, out);
   return cudaGetLastError();
 }
 

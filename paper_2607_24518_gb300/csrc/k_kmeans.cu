@@ -23,33 +23,16 @@
 namespace symnmf {
 namespace {
 
+// ||s_i|| in FP64: one warp per row, runs of 64 entries as float-float sums
 template <int DT>
-__device__ __forceinline__ double s_at(const void *S, int64_t idx) {
-  if constexpr (DT == 0) {
-    return (double)reinterpret_cast<const float *>(S)[idx];
-  } else if constexpr (DT == 1) {
-    return (double)__bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(S)[idx]);
-  } else {
-    __nv_fp8_e4m3 q;
-    q.__x = reinterpret_cast<const __nv_fp8_storage_t *>(S)[idx];
-    return (double)static_cast<float>(q);
-  }
-}
-
-// ||s_i|| in FP64: one warp per row, lanes over columns, xor tree
-template <int DT>
-__global__ void __launch_bounds__(256) row_norms_kernel(const void *S, int64_t n, int64_t lds,
+__global__ void __launch_bounds__(256, 4) row_norms_kernel(const void *S, int64_t n, int64_t lds,
                                                         const float *scales, int64_t ld_scales,
-                                                        double *rn) {
+                                                        bool vec, double *rn) {
   const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= n) return;
-  double acc = 0.0;
-  for (int64_t c = lane; c < n; c += 32) {
-    double v = s_at<DT>(S, row * lds + c);
-    if constexpr (DT == 2) v *= (double)scales[(row / kTileRows) * ld_scales + c / kTileRows];
-    acc += v * v;
-  }
+  double acc =
+      row_sumsq_lane<DT>(S, row * lds, n, scales + (row / kTileRows) * ld_scales, vec, lane);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane == 0) rn[row] = sqrt(acc);
@@ -202,10 +185,11 @@ __global__ void __launch_bounds__(256) km_final_kernel(KmArgs a) {
 cudaError_t launch_row_norms(const void *S, int64_t n, int64_t lds, int dtype, const float *scales,
                              int64_t ld_scales, double *rn, cudaStream_t s) {
   const unsigned blocks = (unsigned)((n + 7) / 8);
+  const bool vec = rows_on_16(S, lds, dtype);
   switch (dtype) {
-    case 0: row_norms_kernel<0><<<blocks, 256, 0, s>>>(S, n, lds, scales, ld_scales, rn); break;
-    case 1: row_norms_kernel<1><<<blocks, 256, 0, s>>>(S, n, lds, scales, ld_scales, rn); break;
-    case 2: row_norms_kernel<2><<<blocks, 256, 0, s>>>(S, n, lds, scales, ld_scales, rn); break;
+    case 0: row_norms_kernel<0><<<blocks, 256, 0, s>>>(S, n, lds, scales, ld_scales, vec, rn); break;
+    case 1: row_norms_kernel<1><<<blocks, 256, 0, s>>>(S, n, lds, scales, ld_scales, vec, rn); break;
+    case 2: row_norms_kernel<2><<<blocks, 256, 0, s>>>(S, n, lds, scales, ld_scales, vec, rn); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

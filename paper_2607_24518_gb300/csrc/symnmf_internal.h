@@ -44,6 +44,12 @@ __host__ __device__ inline float *bt_deq(void *Bt, int kp, int64_t ldb) {
   return reinterpret_cast<float *>(reinterpret_cast<uint8_t *>(Bt) + (size_t)2 * kp * ldb);
 }
 
+// every row of S starts on a 16-byte boundary
+inline bool rows_on_16(const void *S, int64_t lds, int dtype) {
+  const int64_t es = dtype == 0 ? 4 : dtype == 1 ? 2 : 1;
+  return reinterpret_cast<uintptr_t>(S) % 16 == 0 && lds * es % 16 == 0;
+}
+
 constexpr int kRing = 1024;  // device record ring (iterations)
 
 enum Mode : int { MODE_FULL = 0, MODE_ROWS = 1, MODE_BLOCK = 2, MODE_GRAD_ONLY = 3 };
