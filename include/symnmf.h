@@ -421,11 +421,12 @@ int symnmf_set_matrix(symnmf_t h, const void *S, int64_t lds, const float *scale
  * and in FP64 across runs (relative error below 32 * 2^-24).  stream: cudaStream_t as void* (NULL =
  * legacy default); the call synchronises it once at the end.
  * Arithmetic: the centred values are FP32; G is formed on the tensor cores
- * from tf32 hi / lo pieces of each value (hi hi + hi lo + lo hi, FP32
- * accumulation), about FP32 accuracy; column norms are FP64.  A column with
+ * from FP16 hi / lo pieces of each value, scaled by a power of two per column
+ * (22 bits; hi hi + hi lo + lo hi, FP32 accumulation), about FP32 accuracy;
+ * column norms are FP64.  A column with
  * zero variance gives a zero row and column in S except S_ii = 1.
- * Scratch: n (8 T' + 12) + ceil(n/128) ceil(n/256) 8 bytes of stream-ordered
- * device memory (T' = T rounded up to 32), freed before return.
+ * Scratch: n (4 T' + 4) bytes and 8 per SM of stream-ordered device memory
+ * (T' = T rounded up to 32), freed before return.
  * Errors: INVALID for null pointers, T < 1 (T < 2 with center), n < 1,
  * pitches below n, a misaligned S or pitch, an unknown out_dtype, or FP8
  * without scales or with ld_scales < ceil(n/128); UNSUPPORTED for n above
