@@ -95,10 +95,16 @@ struct Cfg {
   static constexpr bool SLO16 = F32 && KP <= 32;
   static constexpr int N2 = SLO16 ? (KP < 16 ? 16 : KP) : 0;
   static constexpr int N = 2 * KP;  // rows of the staged B: [H_hi | H_lo]
-  // FP8 from kp = 16: S H_hi and S H_lo accumulate into one accumulator
-  // (two MMAs of N = kp); kp = 8 keeps one MMA of N = 16 (M = 128 needs N
-  // a multiple of 16) and adds the two parts when folding
-  static constexpr bool JOIN = F8 && KP >= 16;
+  // S H_hi and S H_lo in one accumulator (two MMAs of N = kp), so that the
+  // folders read kp columns per fold instead of 2 kp: FP8 from kp = 16 (kp =
+  // 8 keeps one MMA of N = 16, as M = 128 needs N a multiple of 16, and adds
+  // the two parts when folding) and FP32 at kp = 64, where S_lo H_hi joins
+  // them.  FP32 chains the lo products first: the accumulator is near 2^-11
+  // of its final size then, so the truncation of the chained additions counts
+  // for the hi products alone, as with separate accumulators (step kernel at
+  // n = 30000, k = 64: 1430 -> 1362 us).  BF16 is at the HBM rate either way
+  // (joined: n = 20000, k = 32 142 -> 145 us).
+  static constexpr bool JOIN = F32 ? KP == 64 : F8 && KP >= 16;
   static constexpr int NA = JOIN ? KP : N;  // accumulator columns of the main product
   static constexpr int ATOM_COLS = F32 ? 32 : F8 ? 128 : 64;  // elements per 128-byte row
   static constexpr int APS = (KP == 64 || F8) ? 1 : 2;    // swizzle atoms per stage
@@ -126,7 +132,7 @@ struct Cfg {
   // fewer stages than fit measured faster at kp = 64 (every storage type)
   // and with FP8 at kp = 32: about 120-130 KB in flight per SM; more only
   // lengthens the round trips
-  static constexpr int STAGE_CAP = KP == 64 ? 4 : (F8 && KP == 32) ? 5 : 8;
+    static constexpr int STAGE_CAP = KP == 64 ? 4 : (F8 && KP == 32) ? 5 : 8;
   static constexpr int STAGES = (BUDGET / STAGE) < (uint32_t)STAGE_CAP ? (int)(BUDGET / STAGE) : STAGE_CAP;
   static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE + BAR_BYTES + EPI_BYTES;
   // MMA issuing threads (warps 1 and 14).  One thread issues a tcgen05.mma
@@ -145,15 +151,17 @@ struct Cfg {
   static constexpr uint32_t ACC0 = F32 ? NABUF * ABUF : 0u;
   static constexpr uint32_t ACCW = NA + NL;               // columns per accumulator buffer
   static constexpr uint32_t PB0 = ACC0 + 2 * ACCW;        // double-buffered P rows
-  // kp = 64: the folders keep the running sum of a tile segment in tensor
-  // memory (PA) instead of 64 registers per thread, which the 128-register
-  // budget of a 16-warp CTA cannot hold next to a fold's loads
+  // kp = 64: the folders of BF16 and FP32 storage keep the running sum of a
+  // tile segment, or half of it, in tensor memory (PA) instead of 64
+  // registers per thread, which the 128-register budget of a 16-warp CTA
+  // cannot hold next to a fold's loads of two accumulators or the conversion
   static constexpr bool PTMEM = (KP == 64);
   static constexpr uint32_t PA0 = PB0 + 2 * KP;
-  // columns of the running sum kept in registers (kp = 64 with FP32
-  // storage: half of them, which measured faster there; BF16 and FP8 keep
-  // all of them in PA)
-  static constexpr int NPR = !PTMEM ? KP : F32 ? KP / 2 : 0;
+  // columns of the running sum kept in registers: with FP8, whose joined
+  // accumulator is all a fold reads, every one of them (step kernel at n =
+  // 20000, k = 64: 155 -> 144 us); FP32 half (1417 -> 1362 us at n = 30000),
+  // BF16 none (204 us either way)
+  static constexpr int NPR = !PTMEM || F8 ? KP : F32 ? KP / 2 : 0;
   static constexpr uint32_t TMEM_NEED = PA0 + (uint32_t)(KP - NPR);
   static constexpr uint32_t TMEM_COLS = TMEM_NEED <= 32 ? 32 : TMEM_NEED <= 64 ? 64 : TMEM_NEED <= 128 ? 128 : TMEM_NEED <= 256 ? 256 : 512;
   static_assert(STAGES >= 2, "shared memory ring too small");
@@ -1346,8 +1354,9 @@ __device__ __noinline__ void mma_role(const TcArgs &a, const Segs &sg, uint8_t *
   constexpr int STAGES = C::STAGES;
   constexpr int N = C::N;
   constexpr int FOLD = C::FOLD;
-  constexpr uint32_t idesc =
-      C::F32 ? idesc_tf32(128, N) : C::F8 ? idesc_e4m3(128, C::NA) : idesc_bf16(128, N);
+  constexpr uint32_t idesc = C::F32  ? idesc_tf32(128, C::NA)
+                             : C::F8 ? idesc_e4m3(128, C::NA)
+                                     : idesc_bf16(128, C::NA);
   constexpr uint64_t kLoD = (uint64_t)(KP * 128) >> 4;  // H_lo rows of the staged B
   // descriptor units are 16 bytes; stage, atom and 32-byte K-slice offsets
   constexpr uint64_t kStageD = C::STAGE >> 4, kAtomD = kAtomBytes >> 4, kBAtomD = C::B_ATOM >> 4;
@@ -1375,9 +1384,13 @@ __device__ __noinline__ void mma_role(const TcArgs &a, const Segs &sg, uint8_t *
       break;
     }
     const uint32_t d = tmem_base + C::ACC0 + (uint32_t)acc * C::ACCW;
-#pragma unroll
-    for (int t = 0; t < FOLD; ++t, ++g) {
-      if (!mbar_wait(&full[stage], phase, abort_flag)) {
+    if constexpr (C::F32 && C::JOIN) {
+      // one stage per chain: S H_lo and S_lo H_hi (S_lo from tensor memory,
+      // once the converter warps have stored it), then S H_hi
+      static_assert(FOLD == 1, "one stage per chain");
+      const int ab = (int)(g % C::NABUF);
+      if (!mbar_wait(&full[stage], phase, abort_flag) ||
+          !mbar_wait(&afull[ab], (uint32_t)((g / C::NABUF) & 1), abort_flag)) {
         set_err(a.err, 3);
         ok = false;
         break;
@@ -1385,35 +1398,60 @@ __device__ __noinline__ void mma_role(const TcArgs &a, const Segs &sg, uint8_t *
       fence_after();
       const uint64_t ad = ad_base + (uint64_t)stage * kStageD;
       const uint64_t bd = ad + (C::A_BYTES >> 4);
-      const uint32_t first = (t == 0) ? 0u : 1u;
 #pragma unroll
-      for (int j = 0; j < C::KSL; ++j) {
-        const uint64_t off = (uint64_t)(j & 3) * 2u;  // 32-byte K slice within a 128-byte row
-        const uint64_t adj = ad + (uint64_t)(j >> 2) * kAtomD + off;
-        const uint64_t bdj = bd + (uint64_t)(j >> 2) * kBAtomD + off;
-        const uint32_t accum = (j == 0) ? first : 1u;
-        if constexpr (C::F32) {
-          mma_tf32_ss(d, adj, bdj, idesc, accum);
-        } else if constexpr (C::F8) {
-          mma_e4m3(d, adj, bdj, idesc, accum);
-          if constexpr (C::JOIN) mma_e4m3(d, adj, bdj + kLoD, idesc, 1u);
-        } else {
-          mma_bf16(d, adj, bdj, idesc, accum);
-        }
+      for (int j = 0; j < C::KSL; ++j)
+        mma_tf32_ss(d, ad + (uint64_t)j * 2u, bd + kLoD + (uint64_t)j * 2u, idesc, j == 0 ? 0u : 1u);
+#pragma unroll
+      for (int j = 0; j < C::KSL; ++j)
+        mma_tf32_ta(d, tmem_base + (uint32_t)ab * C::ABUF + (uint32_t)j * 8u, bd + (uint64_t)j * 2u,
+                    idesc, 1u);
+      mma_commit(&aempty[ab]);
+#pragma unroll
+      for (int j = 0; j < C::KSL; ++j)
+        mma_tf32_ss(d, ad + (uint64_t)j * 2u, bd + (uint64_t)j * 2u, idesc, 1u);
+      mma_commit(&empty[stage]);
+      ++g;
+      if (++stage == STAGES) {
+        stage = 0;
+        phase ^= 1u;
       }
-      if constexpr (C::F32) {
-        // S_lo H once the converter warps have stored S_lo in TMEM: as
-        // kind::f16 against bf16(H) (kp <= 32), else as tf32 against H_hi
-        // into the H_lo part
-        const int ab = C::SLO16 ? stage : (int)(g % C::NABUF);
-        const uint32_t aparity = C::SLO16 ? phase : (uint32_t)((g / C::NABUF) & 1);
-        if (!mbar_wait(&afull[ab], aparity, abort_flag)) {
+    } else {
+#pragma unroll
+      for (int t = 0; t < FOLD; ++t, ++g) {
+        if (!mbar_wait(&full[stage], phase, abort_flag)) {
           set_err(a.err, 3);
           ok = false;
           break;
         }
         fence_after();
-        if constexpr (C::SLO16) {
+        const uint64_t ad = ad_base + (uint64_t)stage * kStageD;
+        const uint64_t bd = ad + (C::A_BYTES >> 4);
+        const uint32_t first = (t == 0) ? 0u : 1u;
+#pragma unroll
+        for (int j = 0; j < C::KSL; ++j) {
+          const uint64_t off = (uint64_t)(j & 3) * 2u;  // 32-byte K slice within a 128-byte row
+          const uint64_t adj = ad + (uint64_t)(j >> 2) * kAtomD + off;
+          const uint64_t bdj = bd + (uint64_t)(j >> 2) * kBAtomD + off;
+          const uint32_t accum = (j == 0) ? first : 1u;
+          if constexpr (C::F32) {
+            mma_tf32_ss(d, adj, bdj, idesc, accum);
+          } else if constexpr (C::F8) {
+            mma_e4m3(d, adj, bdj, idesc, accum);
+            if constexpr (C::JOIN) mma_e4m3(d, adj, bdj + kLoD, idesc, 1u);
+          } else {
+            mma_bf16(d, adj, bdj, idesc, accum);
+          }
+        }
+        if constexpr (C::F32) {
+          // S_lo H once the converter warps have stored S_lo in TMEM, as
+          // kind::f16 against bf16(H) into its own accumulator
+          const int ab = stage;
+          if (!mbar_wait(&afull[ab], phase, abort_flag)) {
+            set_err(a.err, 3);
+            ok = false;
+            break;
+          }
+          fence_after();
           constexpr uint32_t idesc16 = idesc_bf16(128, C::N2);
           const uint64_t bd2 = bd + (C::B_BYTES >> 4);
 #pragma unroll
@@ -1421,21 +1459,12 @@ __device__ __noinline__ void mma_role(const TcArgs &a, const Segs &sg, uint8_t *
             const uint32_t alo = tmem_base + (uint32_t)ab * C::ABUF + (uint32_t)j * 8u;
             mma_bf16_ta(d + N, alo, bd2 + (uint64_t)j * 2u, idesc16, (j == 0) ? first : 1u);
           }
-        } else {
-          constexpr uint32_t idesc_lo = idesc_tf32(128, KP >= 16 ? KP : N);
-#pragma unroll
-          for (int j = 0; j < C::KSL; ++j) {
-            const uint64_t bdj = bd + (uint64_t)(j >> 2) * kBAtomD + (uint64_t)(j & 3) * 2u;
-            const uint32_t alo = tmem_base + (uint32_t)ab * C::ABUF + (uint32_t)j * 8u;
-            mma_tf32_ta(d + (KP >= 16 ? KP : 0), alo, bdj, idesc_lo, 1u);
-          }
-          mma_commit(&aempty[ab]);
         }
-      }
-      mma_commit(&empty[stage]);
-      if (++stage == STAGES) {
-        stage = 0;
-        phase ^= 1u;
+        mma_commit(&empty[stage]);
+        if (++stage == STAGES) {
+          stage = 0;
+          phase ^= 1u;
+        }
       }
     }
     if (!ok) break;
