@@ -75,10 +75,7 @@ struct symnmf_ctx {
   double *norm_parts = nullptr;
   int n_norm_parts = 0;
   int *dev_err = nullptr;     // device error word (bounded-wait timeouts)
-  int *counters = nullptr;    // reduction last-arriver counters
   int *tile_cnt = nullptr;    // per-tile stream-K arrival counters
-  double *lvl1 = nullptr;     // reduction level-1 sums
-  int ntc = 0;                // tile chunks of 32
   int *host_err = nullptr;    // pinned mirror
   // host state
   symnmf_ctrl ctrl{};
@@ -170,8 +167,8 @@ void free_all(symnmf_t h) {
                   (void *)h->P, (void *)h->Q, (void *)h->R, (void *)h->slots, (void *)h->chunk,
                   (void *)h->gramI, (void *)h->gramJ, (void *)h->minv, (void *)h->dlists, (void *)h->ring,
                   (void *)h->hist, (void *)h->sel, (void *)h->dmed, (void *)h->dsum,
-                  (void *)h->norm_parts, (void *)h->dev_err, (void *)h->counters, (void *)h->tile_cnt,
-                  (void *)h->lvl1, (void *)h->km_rn, (void *)h->km_lab, (void *)h->km_colsq,
+                  (void *)h->norm_parts, (void *)h->dev_err, (void *)h->tile_cnt,
+                  (void *)h->km_rn, (void *)h->km_lab, (void *)h->km_colsq,
                   (void *)h->km_inv, (void *)h->km_slots, (void *)h->km_out, (void *)h->rs_part,
                   (void *)h->rs_out})
     cudaFree(p);
@@ -226,8 +223,6 @@ ReduceArgs reduce_args(symnmf_t h, const double *slots, const float *gram_part, 
   r.gram64_next = h->gram64[1 - h->cur];
   r.gram32_next = h->gram32[1 - h->cur];
   r.rec = h->ring + (t >= 0 ? (t % kRing) : kRing);
-  r.lvl1 = h->lvl1;
-  r.counters = h->counters;
   return r;
 }
 
@@ -968,10 +963,7 @@ int symnmf_create_ld(const void *S, int64_t n, int64_t lds, int32_t k, int32_t d
   if (e == cudaSuccess) e = dalloc(&h->dsum, 4);
   if (e == cudaSuccess) e = dalloc(&h->norm_parts, (size_t)h->n_norm_parts);
   if (e == cudaSuccess) e = dalloc(&h->dev_err, 4);
-  h->ntc = (h->ntiles + 31) / 32;
-  if (e == cudaSuccess) e = dalloc(&h->counters, 64);
   if (e == cudaSuccess) e = dalloc(&h->tile_cnt, (size_t)h->ntiles);
-  if (e == cudaSuccess) e = dalloc(&h->lvl1, (size_t)h->ntc * (4 + h->kp * h->kp));
   if (e == cudaSuccess) e = cudaMallocHost((void **)&h->host_err, sizeof(int) * 4);
   if (e == cudaSuccess) e = cudaMallocHost((void **)&h->hlists, sizeof(int) * kStages * kListArrays * h->ntiles);
   if (e == cudaSuccess) e = cudaMallocHost((void **)&h->hring, sizeof(DevRecord) * (kRing + 1));
@@ -1200,7 +1192,6 @@ int symnmf_set_H(symnmf_t h, const float *H) {
   CK(cudaMemsetAsync(h->M, 0, bytes, h->stream));
   CK(cudaMemsetAsync(h->mu, 0, bytes, h->stream));
   CK(cudaMemsetAsync(h->g, 0, bytes, h->stream));
-  CK(cudaMemsetAsync(h->counters, 0, sizeof(int) * 64, h->stream));
   CK(cudaMemsetAsync(h->tile_cnt, 0, sizeof(int) * h->ntiles, h->stream));
   reset_ctrl(&h->ctrl);
   reset_restart_checks(h);

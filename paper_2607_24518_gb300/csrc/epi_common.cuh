@@ -254,36 +254,4 @@ __device__ __forceinline__ double row_sumsq_lane(const void *S, int64_t rowbase,
   return acc;
 }
 
-// Sum, in index order, `count` (<= 32) values at base[i * stride]; every
-// load is issued before the ordered additions.
-template <typename T>
-__device__ __forceinline__ double ordered_sum32(const T *base, int64_t stride, int count) {
-  double v[32];
-#pragma unroll
-  for (int j = 0; j < 32; ++j) v[j] = (j < count) ? (double)base[(int64_t)j * stride] : 0.0;
-  double s = 0.0;
-#pragma unroll
-  for (int j = 0; j < 32; ++j) s += v[j];
-  return s;
-}
-
-// Fixed-order sum over nthr threads (et = 0..nthr-1): xor tree inside each
-// warp, then warp partials added in warp order.  scratch holds >= 33
-// doubles; bar() synchronises the participating threads.
-template <class Bar>
-__device__ __forceinline__ double group_sum(double v, int et, int nthr, Bar bar, double *scratch) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  bar();
-  if ((et & 31) == 0) scratch[et >> 5] = v;
-  bar();
-  if (et == 0) {
-    double r = 0.0;
-    for (int i = 0; i < (nthr >> 5); ++i) r += scratch[i];
-    scratch[32] = r;
-  }
-  bar();
-  return scratch[32];
-}
-
 }  // namespace symnmf

@@ -151,8 +151,6 @@ struct ReduceArgs {
   double *gram64_next;
   float *gram32_next;
   DevRecord *rec;            // record destination or nullptr
-  double *lvl1;              // ceil(ntiles/32) x (4 + kp^2) scratch
-  int *counters;             // >= ceil((4 + kp^2)/128) counters, zero between launches
   int kb;                    // restarts along N: Gram entries whose columns lie in
                              // different blocks of kb columns are set to 0 (0: none)
 };
