@@ -388,10 +388,8 @@ int prod(symnmf_t h, const int *row_list, int n_rows, const int *col_list, int n
   a.col_list = col_list;
   a.n_cols_list = n_cols;
   a.out = out;
-  const int target = 3 * h->num_sms;
-  int ns = (target + n_rows - 1) / std::max(1, n_rows);
-  ns = std::max(1, std::min(ns, std::min(64, n_cols)));
-  if ((int64_t)ns * n_rows > h->pq_cap_tiles) ns = (int)std::max<int64_t>(1, h->pq_cap_tiles / n_rows);
+  const int64_t most = std::min<int64_t>(64, h->pq_cap_tiles / std::max(1, n_rows));
+  const int ns = simt_shares(n_rows, n_cols, h->num_sms, (int)std::max<int64_t>(1, most));
   a.nsplit = ns;
   lay->nsplit = ns;
   lay->skG = 0;

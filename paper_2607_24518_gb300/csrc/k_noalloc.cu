@@ -11,41 +11,26 @@
 //
 // Three kernels: (1) one CTA per (row tile, column share) multiplies its
 // share of S by H (FP32 FMA) and immediately dots the partial product rows
-// with H_I, leaving one FP64 partial of tr per CTA; (2) one CTA per row
-// tile writes the FP32 Gram partial H_I^T H_I; (3) one CTA adds the
-// partials in a fixed order in FP64 and writes f.  Every scratch slot that
-// (3) reads is written by (1) or (2) earlier in the same call, so nothing
-// in the scratch has to start at zero, and two calls with the same inputs
-// give the same bits.
-#include <cuda_bf16.h>
-#include <cuda_fp8.h>
-
+// with H_I, leaving one FP64 partial of tr per CTA, and one more CTA per row
+// tile writes the FP32 Gram partial H_I^T H_I; (2) 16 Gram entries per CTA
+// are added across tiles in FP64, leaving the sum of their squares; (3) one
+// CTA adds the partials in a fixed order in FP64 and writes f.  Every scratch
+// slot that is read is written earlier in the same call, so nothing in the
+// scratch has to start at zero, and two calls with the same inputs give the
+// same bits.
 #include <mutex>
 
 #include "../../include/symnmf.h"
+#include "simt_tile.cuh"
 #include "symnmf_internal.h"
 
 namespace symnmf {
 namespace {
 
-constexpr int kSplit = 8;   // column shares per row tile in kernel (1)
-constexpr int BK = 32;
+constexpr int kSplit = 8;   // at most so many column shares per row tile in kernel (1)
 constexpr int kMaxDevices = 64;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[SYMNMF_NOALLOC_SCRATCH_BYTES];
-
-template <int DT>
-__device__ __forceinline__ float load_s(const void *S, int64_t idx) {
-  if constexpr (DT == 0) {
-    return __ldg(reinterpret_cast<const float *>(S) + idx);
-  } else if constexpr (DT == 1) {
-    return __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(S)[idx]);
-  } else {
-    __nv_fp8_e4m3 q;
-    q.__x = reinterpret_cast<const __nv_fp8_storage_t *>(S)[idx];
-    return static_cast<float>(q);
-  }
-}
 
 struct ObjArgs {
   const void *S;
@@ -56,8 +41,12 @@ struct ObjArgs {
   int k;
   int ntiles;
   double normS2;
-  double *tr_part;  // ntiles * kSplit
+  int split;        // column shares per row tile, at most kSplit
+  double *tr_part;  // ntiles * kSplit; slot [tile * kSplit + split] of a share
   float *gram_part; // ntiles * kp * kp
+  // the CTA sums of squares of kernel (2): CTA b's over its own entries 16 b
+  // and 16 b + 1 of tile 0's Gram partial, which it alone has read by then
+  __device__ double *g2_slot(int b) const { return reinterpret_cast<double *>(gram_part + 16 * b); }
   double *f;
 };
 
@@ -75,86 +64,78 @@ __device__ __forceinline__ double block_sum_fixed(double v, double *sh) {
   return r;  // valid in thread 0
 }
 
+// the Gram partial of a row tile: rows r = 4 i + g in four FMA chains, added
+// (s0 + s1) + (s2 + s3), the row order of the solver's Gram partials
+template <int KP>
+__device__ void gram_tile(const ObjArgs &a, int tile, float *sm) {
+  float(*Hn)[KP + 1] = reinterpret_cast<float(*)[KP + 1]>(sm);
+  const int64_t r0 = (int64_t)tile * kTileRows;
+  for (int e = threadIdx.x; e < kTileRows * KP; e += 256) {
+    const int r = e / KP, c = e % KP;
+    Hn[r][c] = (r0 + r < a.n && c < a.k) ? a.H[(r0 + r) * a.k + c] : 0.f;
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < KP * KP; q += 256)
+    a.gram_part[(int64_t)tile * KP * KP + q] = gram_entry<KP>(Hn, q / KP, q % KP);
+}
+
+// blockIdx.y < split: a column share; == split: the tile's Gram partial.
+// n = 10000, KP = 32 FP32: 500 -> 244 us (13 TFMA/s of 37); the tile Grams
+// beside the shares and their sum over the chip replace a pass of their own
+// and one CTA's 49 us.
 template <int DT, int KP>
-__global__ void __launch_bounds__(256) tr_share_kernel(ObjArgs a) {
-  constexpr int CG = KP / 4, RG = 256 / CG, TM = 128 / RG;
-  __shared__ float Ss[128][BK + 1];
-  __shared__ __align__(16) float Hs[BK][KP];
+__global__ void __launch_bounds__(256, 2) tr_share_kernel(ObjArgs a) {
+  extern __shared__ __align__(16) float sm_obj[];
   __shared__ double red[8];
   const int tid = threadIdx.x, tile = blockIdx.x, split = blockIdx.y;
-  const int64_t r0 = (int64_t)tile * kTileRows;
-  const int per = (a.ntiles + kSplit - 1) / kSplit;
-  const int cb = split * per, ce = min(a.ntiles, cb + per);
-  const int cg = tid % CG, rg = tid / CG;
-  float acc[TM][4];
-#pragma unroll
-  for (int i = 0; i < TM; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
-  for (int ct = cb; ct < ce; ++ct) {
-    const int64_t c0 = (int64_t)ct * kTileRows;
-    float scale = 1.f;
-    if constexpr (DT == 2) scale = a.scales[(int64_t)tile * a.ld_scales + ct];
-    for (int kk = 0; kk < kTileRows; kk += BK) {
-      for (int e = tid; e < 128 * BK; e += 256) {
-        const int r = e / BK, c = e % BK;
-        const int64_t gr = r0 + r, gc = c0 + kk + c;
-        Ss[r][c] = (gr < a.n && gc < a.n) ? load_s<DT>(a.S, gr * a.lds + gc) * scale : 0.f;
-      }
-      for (int e = tid; e < BK * KP; e += 256) {
-        const int r = e / KP, c = e % KP;
-        const int64_t gr = c0 + kk + r;
-        Hs[r][c] = (gr < a.n && c < a.k) ? a.H[gr * a.k + c] : 0.f;
-      }
-      __syncthreads();
-#pragma unroll 8
-      for (int x = 0; x < BK; ++x) {
-        const float4 hv = *reinterpret_cast<const float4 *>(&Hs[x][cg * 4]);
-#pragma unroll
-        for (int i = 0; i < TM; ++i) {
-          const float sv = Ss[rg + i * RG][x];
-          acc[i][0] = fmaf(sv, hv.x, acc[i][0]);
-          acc[i][1] = fmaf(sv, hv.y, acc[i][1]);
-          acc[i][2] = fmaf(sv, hv.z, acc[i][2]);
-          acc[i][3] = fmaf(sv, hv.w, acc[i][3]);
-        }
-      }
-      __syncthreads();
-    }
+  if (split == a.split) {
+    gram_tile<KP>(a, tile, sm_obj);
+    return;
   }
+  const int64_t r0 = (int64_t)tile * kTileRows;
+  const int per = (a.ntiles + a.split - 1) / a.split;
+  const int cb = min(a.ntiles, split * per), ce = min(a.ntiles, cb + per);
+  simt_tile<DT, KP>(sm_obj, a.S, a.lds, a.n, r0, a.H, a.k, a.k, nullptr, cb, ce,
+                    DT == 2 ? a.scales + (int64_t)tile * a.ld_scales : nullptr);
   // this share's part of sum_{r, c} H_rc (S H)_rc over the tile's rows
   float t = 0.f;
-#pragma unroll
-  for (int i = 0; i < TM; ++i) {
-    const int64_t gr = r0 + rg + i * RG;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = cg * 4 + j;
-      if (gr < a.n && c < a.k) t = fmaf(a.H[gr * a.k + c], acc[i][j], t);
-    }
+#pragma unroll 4
+  for (int e = tid; e < kTileRows * KP; e += 256) {
+    const int r = e / KP, c = e % KP;
+    if (r0 + r < a.n && c < a.k) t = fmaf(__ldg(a.H + (r0 + r) * a.k + c), sm_obj[e], t);
   }
   const double s = block_sum_fixed((double)t, red);
   if (tid == 0) a.tr_part[(int64_t)tile * kSplit + split] = s;
 }
 
+// 16 Gram entries per CTA, 16 threads to an entry: tiles j, j + 16, ... in
+// order, then the 16 sums in order; the sum of the entries' squares goes to
+// the CTA's g2_slot
 template <int KP>
-__global__ void __launch_bounds__(256) gram_tile_kernel(ObjArgs a) {
-  __shared__ float Hn[kTileRows][KP + 1];
-  const int tile = blockIdx.x;
-  const int64_t r0 = (int64_t)tile * kTileRows;
-  for (int e = threadIdx.x; e < kTileRows * KP; e += blockDim.x) {
-    const int r = e / KP, c = e % KP;
-    Hn[r][c] = (r0 + r < a.n && c < a.k) ? a.H[(r0 + r) * a.k + c] : 0.f;
-  }
-  __syncthreads();
-  for (int q = threadIdx.x; q < KP * KP; q += blockDim.x) {
-    // rows r = 4 i + g in four FMA chains, added (s0 + s1) + (s2 + s3): the
-    // row order of the solver's Gram partials
-    const int c = q / KP, d = q % KP;
-    float s[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-    for (int i = 0; i < kTileRows / 4; ++i)
+__global__ void __launch_bounds__(256) gram_sum_kernel(ObjArgs a) {
+  __shared__ double red[256];
+  const int tid = threadIdx.x, le = tid & 15, j = tid >> 4;
+  const float *src = a.gram_part + blockIdx.x * 16 + le;
+  double v = 0.0;
+  for (int t0 = j; t0 < a.ntiles; t0 += 128) {
+    float x[8];
 #pragma unroll
-      for (int g = 0; g < 4; ++g) s[g] = fmaf(Hn[4 * i + g][c], Hn[4 * i + g][d], s[g]);
-    a.gram_part[(int64_t)tile * KP * KP + q] = (s[0] + s[1]) + (s[2] + s[3]);
+    for (int u = 0; u < 8; ++u)
+      x[u] = t0 + 16 * u < a.ntiles ? __ldcg(src + (int64_t)(t0 + 16 * u) * KP * KP) : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (t0 + 16 * u < a.ntiles) v += (double)x[u];
+  }
+  red[tid] = v;
+  __syncthreads();
+  if (tid < 16) {
+    double g = 0.0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) g += red[i * 16 + tid];
+    g *= g;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffu, g, o);
+    if (tid == 0) *a.g2_slot(blockIdx.x) = g;
   }
 }
 
@@ -162,18 +143,13 @@ template <int KP>
 __global__ void __launch_bounds__(256) finish_kernel(ObjArgs a) {
   __shared__ double red[8];
   const int tid = threadIdx.x;
-  // tr: thread tid adds a contiguous run of partials, runs added in order
-  const int64_t m = (int64_t)a.ntiles * kSplit;
-  const int64_t per = (m + 255) / 256;
+  // tr: thread tid adds a contiguous run of tiles, runs added in order
+  const int per = (a.ntiles + 255) / 256;
   double tr = 0.0;
-  for (int64_t i = tid * per; i < m && i < (tid + 1) * per; ++i) tr += a.tr_part[i];
-  // ||H^T H||^2: each Gram entry summed over tiles in tile order
+  for (int t = tid * per; t < a.ntiles && t < (tid + 1) * per; ++t)
+    for (int s = 0; s < a.split; ++s) tr += a.tr_part[(int64_t)t * kSplit + s];
   double g2 = 0.0;
-  for (int q = tid; q < KP * KP; q += 256) {
-    double g = 0.0;
-    for (int t = 0; t < a.ntiles; ++t) g += (double)a.gram_part[(int64_t)t * KP * KP + q];
-    g2 += g * g;
-  }
+  if (tid < KP * KP / 16) g2 = *a.g2_slot(tid);
   const double trs = block_sum_fixed(tr, red);
   const double g2s = block_sum_fixed(g2, red);
   if (tid == 0) *a.f = a.normS2 - 2.0 * trs + g2s;
@@ -181,8 +157,8 @@ __global__ void __launch_bounds__(256) finish_kernel(ObjArgs a) {
 
 template <int DT, int KP>
 cudaError_t launch_all(const ObjArgs &a, cudaStream_t s) {
-  tr_share_kernel<DT, KP><<<dim3(a.ntiles, kSplit), 256, 0, s>>>(a);
-  gram_tile_kernel<KP><<<a.ntiles, 256, 0, s>>>(a);
+  tr_share_kernel<DT, KP><<<dim3(a.ntiles, a.split + 1), 256, Simt<DT, KP>::SMEM, s>>>(a);
+  gram_sum_kernel<KP><<<KP * KP / 16, 256, 0, s>>>(a);
   finish_kernel<KP><<<1, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
@@ -200,24 +176,33 @@ cudaError_t launch_dt(const ObjArgs &a, int kp, cudaStream_t s) {
 
 std::mutex g_addr_mu;
 void *g_addr[kMaxDevices] = {};
+int g_sms[kMaxDevices] = {};
 
 // Load every kernel this entry point launches on the current device.  With
 // lazy module loading each kernel would otherwise be loaded at its first
 // launch, i.e. inside some later call, which may allocate and synchronise.
+// (tr_share also takes more shared memory than a kernel may use by default)
+template <int DT, int KP>
+cudaError_t preload_tr() {
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaFuncGetAttributes(&fa, tr_share_kernel<DT, KP>);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(tr_share_kernel<DT, KP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)Simt<DT, KP>::SMEM);
+  return e;
+}
 template <int DT>
 cudaError_t preload_dt() {
-  cudaFuncAttributes fa;
-  cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, tr_share_kernel<DT, 8>);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, tr_share_kernel<DT, 16>);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, tr_share_kernel<DT, 32>);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, tr_share_kernel<DT, 64>);
+  cudaError_t e = preload_tr<DT, 8>();
+  if (e == cudaSuccess) e = preload_tr<DT, 16>();
+  if (e == cudaSuccess) e = preload_tr<DT, 32>();
+  if (e == cudaSuccess) e = preload_tr<DT, 64>();
   return e;
 }
 template <int KP>
 cudaError_t preload_kp() {
   cudaFuncAttributes fa;
-  cudaError_t e = cudaFuncGetAttributes(&fa, gram_tile_kernel<KP>);
+  cudaError_t e = cudaFuncGetAttributes(&fa, gram_sum_kernel<KP>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, finish_kernel<KP>);
   return e;
 }
@@ -282,6 +267,7 @@ extern "C" int symnmf_objective_noalloc(const void *S, int64_t n, int64_t lds, i
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return SYMNMF_ERR_CUDA;
   void *base = nullptr;
+  int sms = 0;
   {
     // first call on a device: look up that device's copy of the scratch
     // (this loads the library's module there, creating the array) and load
@@ -290,6 +276,7 @@ extern "C" int symnmf_objective_noalloc(const void *S, int64_t n, int64_t lds, i
     if (!g_addr[dev]) {
       void *p = nullptr;
       if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess ||
+          cudaDeviceGetAttribute(&g_sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
           preload_kernels() != cudaSuccess) {
         cudaGetLastError();
         return SYMNMF_ERR_CUDA;
@@ -297,6 +284,7 @@ extern "C" int symnmf_objective_noalloc(const void *S, int64_t n, int64_t lds, i
       g_addr[dev] = p;
     }
     base = g_addr[dev];
+    sms = g_sms[dev];
   }
   ObjArgs a{};
   a.S = S;
@@ -307,6 +295,7 @@ extern "C" int symnmf_objective_noalloc(const void *S, int64_t n, int64_t lds, i
   a.H = H;
   a.k = k;
   a.ntiles = (int)ntiles;
+  a.split = simt_split(a.ntiles, a.ntiles, 2 * sms, kSplit);
   a.normS2 = normS2;
   a.tr_part = reinterpret_cast<double *>(base);
   a.gram_part = reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(base) + tr_bytes);
