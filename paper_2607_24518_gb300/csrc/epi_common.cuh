@@ -92,11 +92,14 @@ __device__ __forceinline__ float part_sum(const float *P, int nsplit, int skG, i
 // num / (sqrt(v) + eps), the AdaGrad / RMSprop step (Sec. 2.2), in
 // straight-line code: PTX sqrt.approx.f32 (relative error at most 2^-23)
 // and div.full.f32 (at most 2 ulp over the full range).  With no
-// out-of-line special-case path the columns of a row overlap in flight.
+// out-of-line special-case path the columns of a row overlap in flight.  The
+// sum, and what callers do with the quotient, are rounded on their own: the
+// assembler may otherwise fuse them with the last multiplication inside the
+// square root or the quotient, in one kernel and not in another.
 __device__ __forceinline__ float adaptive_step(float num, float v, float eps) {
   float r, q;
   asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
-  asm("div.full.f32 %0, %1, %2;" : "=f"(q) : "f"(num), "f"(r + eps));
+  asm("div.full.f32 %0, %1, %2;" : "=f"(q) : "f"(num), "f"(__fadd_rn(r, eps)));
   return q;
 }
 

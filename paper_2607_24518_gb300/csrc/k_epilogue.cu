@@ -40,9 +40,49 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
   return sh[32];
 }
 
+// The Gram partial of the tile in Hn by the T threads of the block, in the
+// row order of every Gram partial: the lanes of a quad hold the four FMA
+// chains of a B x B block of the 8 x 8 block grid (T = 512: of half its
+// rows), so an entry costs two shared-memory reads per B FMAs, not per FMA.
+template <int KP, int T>
+__device__ __forceinline__ void tile_gram(const float (*Hn)[KP + 1], float *gp) {
+  constexpr int B = KP / 8, PARTS = T / 256, BR = B / PARTS;
+  const int part = threadIdx.x >> 8, et = threadIdx.x & 255;
+  const int g = et & 3, bl = (et >> 2) & 7, wq = et >> 5;
+  const int c0 = (2 * (wq >> 1) + (bl >> 2)) * B + part * BR;
+  const int d0 = (4 * (wq & 1) + (bl & 3)) * B;
+  float acc[BR][B];
+#pragma unroll
+  for (int i = 0; i < BR; ++i)
+#pragma unroll
+    for (int j = 0; j < B; ++j) acc[i][j] = 0.f;
+#pragma unroll 4
+  for (int i = 0; i < 32; ++i) {
+    const float *hr = Hn[4 * i + g];
+    float x[BR], y[B];
+#pragma unroll
+    for (int ii = 0; ii < BR; ++ii) x[ii] = hr[c0 + ii];
+#pragma unroll
+    for (int jj = 0; jj < B; ++jj) y[jj] = hr[d0 + jj];
+#pragma unroll
+    for (int ii = 0; ii < BR; ++ii)
+#pragma unroll
+      for (int jj = 0; jj < B; ++jj) acc[ii][jj] = fmaf(x[ii], y[jj], acc[ii][jj]);
+  }
+#pragma unroll
+  for (int ii = 0; ii < BR; ++ii) {
+#pragma unroll
+    for (int jj = 0; jj < B; ++jj) acc[ii][jj] = gram_quad_sum(acc[ii][jj]);
+    if ((ii * 4) / BR == g) {  // the quad's lanes share the stores
+#pragma unroll
+      for (int jj = 0; jj < B; ++jj) gp[(c0 + ii) * KP + d0 + jj] = acc[ii][jj];
+    }
+  }
+}
+
 // writes the transposed MMA copy (format bt_fmt) and the Gram partial of
 // the tile held in smem Hn[128][KP+1]; every thread of the block calls it
-template <int KP>
+template <int KP, int T>
 __device__ void tile_tail(const float (*Hn)[KP + 1], int64_t r0, void *Bt, int bt_fmt, int64_t ldb,
                           float *gram_part, int tile) {
   const int tid = threadIdx.x;
@@ -90,43 +130,98 @@ __device__ void tile_tail(const float (*Hn)[KP + 1], int64_t r0, void *Bt, int b
       B16[(int64_t)c * ldb + r0 + r] = bf16_bits(v);
     }
   }
-  if (gram_part) {
-    for (int q = tid; q < KP * KP; q += blockDim.x)
-      gram_part[(int64_t)tile * KP * KP + q] = gram_entry<KP>(Hn, q / KP, q % KP);
+  if (gram_part) tile_gram<KP, T>(Hn, gram_part + (int64_t)tile * KP * KP);
+}
+
+// A thread's 4 columns (from 4 cg) of RP rows (rg, rg + RS, ...): the rows of
+// a warp's load or store of one of them are contiguous.
+template <int KP>
+struct EpiK {
+  static constexpr int T = KP == 8 ? 256 : 512;
+  static constexpr int CG = KP / 4;
+  static constexpr int RS = T / CG;
+  static constexpr int RP = kTileRows / RS;
+  static constexpr size_t SMEM = sizeof(float) * (kTileRows * (KP + 1) + 3 + 2 * KP * KP);
+};
+
+// acc = (rows of Hs) M for the thread's entries, M (KP x KP) in shared
+// memory, summed over d in order: RP scalar and one 16-byte read per 4 RP FMAs
+template <int KP>
+__device__ __forceinline__ void rows_times(const float (*Hs)[KP + 1], const float *M, int rg,
+                                           int cg, float (&acc)[EpiK<KP>::RP][4]) {
+  constexpr int RP = EpiK<KP>::RP, RS = EpiK<KP>::RS;
+#pragma unroll
+  for (int i = 0; i < RP; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
+#pragma unroll 8
+  for (int d = 0; d < KP; ++d) {
+    const float4 m = *reinterpret_cast<const float4 *>(M + d * KP + 4 * cg);
+#pragma unroll
+    for (int i = 0; i < RP; ++i) {
+      const float h = Hs[rg + i * RS][d];
+      acc[i][0] = fmaf(h, m.x, acc[i][0]);
+      acc[i][1] = fmaf(h, m.y, acc[i][1]);
+      acc[i][2] = fmaf(h, m.z, acc[i][2]);
+      acc[i][3] = fmaf(h, m.w, acc[i][3]);
+    }
   }
 }
 
+// the thread's entries of the summed partials of row position p, slots in
+// order (part_range and part_sum layouts), four loads in flight
 template <int KP>
-constexpr size_t epi_smem_bytes() {
-  return (size_t)(2 * kTileRows * (KP + 1) + 2 * KP * (KP + 1)) * sizeof(float);
+__device__ __forceinline__ void parts_of(const float *P, int nsplit, int skG, int ncols, int nlist,
+                                         int p, int rg, int cg, float (&v)[EpiK<KP>::RP][4]) {
+  constexpr int RP = EpiK<KP>::RP, RS = EpiK<KP>::RS;
+  int64_t b0, b1;
+  part_range(p, skG, ncols, nlist, b0, b1);
+  const int64_t first = skG > 0 ? b0 + p : p, step = skG > 0 ? 1 : nlist;
+  const int count = skG > 0 ? (int)(b1 - b0) + 1 : nsplit;
+#pragma unroll
+  for (int i = 0; i < RP; ++i) {
+    const float *src = P + (first * kTileRows + rg + i * RS) * KP + 4 * cg;
+    const int64_t st = step * kTileRows * KP;
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int q0 = 0; q0 < count; q0 += 4) {
+      float4 x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        x[u] = q0 + u < count ? __ldcg(reinterpret_cast<const float4 *>(src + (q0 + u) * st))
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        s[0] += x[u].x;
+        s[1] += x[u].y;
+        s[2] += x[u].z;
+        s[3] += x[u].w;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[i][j] = s[j];
+  }
 }
 
-constexpr int kEpiThreads = 512;
-
+// Stand-alone tile epilogue, one CTA per 128-row tile.  Bound by latency and
+// shared-memory reads: the H Gram products are formed in 4-column register
+// blocks and the state moves in 16-byte rows.  Multiply-adds are written out,
+// so that every padded rank rounds the same way (restarts in one handle are
+// bit-equal to separate handles).  n = 50000, kp = 64, block mode 337 -> 95
+// us; n = 5001, kp = 32 33 -> 12; n = 3001, kp = 16 19 -> 9.6 (two shared
+// reads per FMA and FP64 block sums before).
 template <int KP>
-__global__ void __launch_bounds__(kEpiThreads) epilogue_kernel(EpiArgs a) {
-  constexpr int EPT = kTileRows * KP / kEpiThreads;  // elements per thread
-  extern __shared__ float smem_epi[];
+__global__ void __launch_bounds__(EpiK<KP>::T, KP == 64 ? 1 : 1024 / EpiK<KP>::T)
+    epilogue_kernel(EpiArgs a) {
+  using K = EpiK<KP>;
+  constexpr int RP = K::RP, RS = K::RS, T = K::T;
+  extern __shared__ __align__(16) float smem_epi[];
   float(*Hs)[KP + 1] = reinterpret_cast<float(*)[KP + 1]>(smem_epi);
-  float(*Hn)[KP + 1] = reinterpret_cast<float(*)[KP + 1]>(smem_epi + kTileRows * (KP + 1));
-  float(*G1)[KP + 1] = reinterpret_cast<float(*)[KP + 1]>(smem_epi + 2 * kTileRows * (KP + 1));
-  float(*G2)[KP + 1] =
-      reinterpret_cast<float(*)[KP + 1]>(smem_epi + 2 * kTileRows * (KP + 1) + KP * (KP + 1));
-  __shared__ double red[40];
+  float *G1 = smem_epi + (kTileRows * (KP + 1) + 3) / 4 * 4, *G2 = G1 + KP * KP;
+  __shared__ double red[T / 32][4];
   const int tile = blockIdx.x, tid = threadIdx.x;
+  const int cg = tid % K::CG, rg = tid / K::CG, c0 = 4 * cg;
   const int64_t r0 = (int64_t)tile * kTileRows;
   const int rows = (int)((a.n - r0) < kTileRows ? (a.n - r0) : kTileRows);
-  const float *__restrict__ Hg = a.H;
-  for (int e = tid; e < kTileRows * KP; e += kEpiThreads) {
-    const int r = e / KP, c = e % KP;
-    Hs[r][c] = (r < rows) ? Hg[(r0 + r) * KP + c] : 0.f;
-  }
   const bool block = (a.mode == MODE_BLOCK);
-  const float *g1src = block ? a.gramJ : a.gram;
-  for (int e = tid; e < KP * KP; e += kEpiThreads) {
-    G1[e / KP][e % KP] = g1src[e];
-    if (block) G2[e / KP][e % KP] = a.gramI[e];
-  }
+  const bool rms = (a.method == SYMNMF_RMSPROP), admm = (a.method == SYMNMF_ADMM);
   int p1 = -1, p2 = -1, p3 = -1;
   if (a.mode == MODE_FULL || a.mode == MODE_GRAD_ONLY) {
     p1 = tile;
@@ -137,165 +232,190 @@ __global__ void __launch_bounds__(kEpiThreads) epilogue_kernel(EpiArgs a) {
       p3 = a.pos3[tile];
     }
   }
-  // block mode: a list whose column list was empty holds no partials
-  const bool has1 = p1 >= 0 && (!block || a.ncols1 > 0);
-  const bool has2 = p2 >= 0 && a.ncols2 > 0;
-  const bool has3 = p3 >= 0 && a.ncols3 > 0;
-  int64_t b10 = 0, b11 = 0, b20 = 0, b21 = 0, b30 = 0, b31 = 0;
-  if (has1 && a.skG1 > 0) {
-    const int64_t W = (int64_t)a.n1 * a.ncols1;
-    b10 = sk_cta((int64_t)p1 * a.ncols1, W, a.skG1);
-    b11 = sk_cta((int64_t)p1 * a.ncols1 + a.ncols1 - 1, W, a.skG1);
-  }
-  if (has2 && a.skG2 > 0) {
-    const int64_t W = (int64_t)a.n2 * a.ncols2;
-    b20 = sk_cta((int64_t)p2 * a.ncols2, W, a.skG2);
-    b21 = sk_cta((int64_t)p2 * a.ncols2 + a.ncols2 - 1, W, a.skG2);
-  }
-  if (has3 && a.skG3 > 0) {
-    const int64_t W = (int64_t)a.n3 * a.ncols3;
-    b30 = sk_cta((int64_t)p3 * a.ncols3, W, a.skG3);
-    b31 = sk_cta((int64_t)p3 * a.ncols3 + a.ncols3 - 1, W, a.skG3);
-  }
-
-  // phase 1: issue every global load of this thread's elements
-  float pv[EPT], qv[EPT], av[EPT], mv[EPT], uv[EPT];
-  const bool rms = (a.method == SYMNMF_RMSPROP);
-  const bool admm = (a.method == SYMNMF_ADMM);
+  const int64_t base = (r0 + rg) * KP + c0;  // entry (i, j): base + i RS KP + j
+  auto ld4 = [&](const float *src, int i) -> float4 {
+    return rg + i * RS < rows ? __ldcg(reinterpret_cast<const float4 *>(src + base + (int64_t)i * RS * KP))
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  auto st4 = [&](float *dst, int i, const float (&x)[4]) {
+    if (rg + i * RS < rows)
+      *reinterpret_cast<float4 *>(dst + base + (int64_t)i * RS * KP) = make_float4(x[0], x[1], x[2], x[3]);
+  };
+  float h[RP][4], g[RP][4], pv[RP][4];
 #pragma unroll
-  for (int i = 0; i < EPT; ++i) {
-    const int e = tid + i * kEpiThreads;
-    const int r = e / KP, c = e % KP;
-    const bool valid = (r < rows) && (c < a.k);
-    const int64_t gi = (r0 + r) * KP + c;
-    pv[i] = (valid && has1)
-                ? part_sum<KP>(a.P, a.nsplit, a.skG1, a.ncols1, a.n1, p1, r, c, b10, b11)
-                : 0.f;
-    qv[i] = (valid && has2)
-                ? part_sum<KP>(a.Q, a.nsplit2, a.skG2, a.ncols2, a.n2, p2, r, c, b20, b21)
-                : 0.f;
-    if (valid && has3) {
-      const float rv = part_sum<KP>(a.R, a.nsplit3, a.skG3, a.ncols3, a.n3, p3, r, c, b30, b31);
-      pv[i] = (p1 >= 0) ? rv + pv[i] : 0.f;
-      qv[i] = (p2 >= 0) ? rv + qv[i] : 0.f;
-    }
-    uv[i] = (valid && p1 < 0 && p2 < 0) ? a.mu[gi] : 0.f;
-    av[i] = (valid && a.update) ? a.A[gi] : 0.f;
-    mv[i] = (valid && a.update && rms) ? a.M[gi] : 0.f;
+  for (int i = 0; i < RP; ++i) {
+    const float4 v = ld4(a.H, i);
+    h[i][0] = v.x;
+    h[i][1] = v.y;
+    h[i][2] = v.z;
+    h[i][3] = v.w;
   }
-  __syncthreads();
+  const float *g1src = block ? a.gramJ : a.gram;
+  for (int e = tid; e < KP * KP / 4; e += T) {
+    reinterpret_cast<float4 *>(G1)[e] = reinterpret_cast<const float4 *>(g1src)[e];
+    if (block) reinterpret_cast<float4 *>(G2)[e] = reinterpret_cast<const float4 *>(a.gramI)[e];
+  }
+#pragma unroll
+  for (int i = 0; i < RP; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      Hs[rg + i * RS][c0 + j] = h[i][j];
+      pv[i][j] = 0.f;
+      g[i][j] = 0.f;
+    }
+  // block mode: a list whose column list was empty holds no partials; list 3
+  // holds what lists 1 and 2 share
+  float rv[RP][4];
+  const bool has3 = p3 >= 0 && a.ncols3 > 0;
+  if (has3) parts_of<KP>(a.R, a.nsplit3, a.skG3, a.ncols3, a.n3, p3, rg, cg, rv);
+  if (p1 >= 0) {
+    if (!block || a.ncols1 > 0)
+      parts_of<KP>(a.P, a.nsplit, a.skG1, a.ncols1, a.n1, p1, rg, cg, pv);
+    if (has3) {
+#pragma unroll
+      for (int i = 0; i < RP; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) pv[i][j] = rv[i][j] + pv[i][j];
+    }
+  }
+  __syncthreads();  // Hs, G1 and G2 are complete
 
-  // phase 2: gradient, update, projection
+  // gradient estimate
   float tr = 0.f, kkt2 = 0.f, sumA = 0.f;
   int nonfin = 0;
+  if (p1 >= 0) {
+    float hg[RP][4];
+    rows_times<KP>(Hs, G1, rg, cg, hg);
 #pragma unroll
-  for (int i = 0; i < EPT; ++i) {
-    const int e = tid + i * kEpiThreads;
-    const int r = e / KP, c = e % KP;
-    float hn = 0.f;
-    if (r < rows && c < a.k) {
-      const int64_t gi = (r0 + r) * KP + c;
-      const float h = Hs[r][c];
-      float g;
-      if (p1 >= 0 || p2 >= 0) {
-        g = 0.f;
-        if (p1 >= 0) {
-          float hg = 0.f;
+    for (int i = 0; i < RP; ++i)
 #pragma unroll
-          for (int d = 0; d < KP; ++d) hg = fmaf(Hs[r][d], G1[d][c], hg);
-          g = a.coef * (hg - pv[i]);
-          tr = fmaf(h, pv[i], tr);
-        }
-        if (p2 >= 0) {
-          float hg = 0.f;
-#pragma unroll
-          for (int d = 0; d < KP; ++d) hg = fmaf(Hs[r][d], G2[d][c], hg);
-          g += a.coef * (hg - qv[i]);
-        }
-      } else {
-        g = uv[i];
+      for (int j = 0; j < 4; ++j) {
+        g[i][j] = __fmul_rn(a.coef, hg[i][j] - pv[i][j]);
+        if (rg + i * RS < rows && c0 + j < a.k) tr = fmaf(h[i][j], pv[i][j], tr);
       }
-      const float pg = (h > 0.f) ? g : fminf(0.f, g);
-      kkt2 = fmaf(pg, pg, kkt2);
-      if (!isfinite(g)) ++nonfin;
-      if (a.gout) a.gout[gi] = g;
-      if (a.gcaller) a.gcaller[(r0 + r) * a.k + c] = g;
-      if (a.store_mu) a.mu[gi] = g;
-      if (a.update && admm) {
-        // ADMM right-hand-side row 2 (S W) + rho (W - U), finished below
-        hn = 2.f * pv[i] + a.rho * (h - av[i]);
-      } else if (a.update) {
-        float x;
-        if (rms) {
-          const float v = a.alpha * av[i] + (1.f - a.alpha) * (g * g);
-          a.A[gi] = v;
-          const float m = a.mom * mv[i] + adaptive_step(a.eta * g, v, a.eps);
-          a.M[gi] = m;
-          x = h - m;
-          sumA += v;
-        } else {
-          const float acc = av[i] + g * g;
-          a.A[gi] = acc;
-          x = h - adaptive_step(a.eta * g, acc, a.eps);
-          sumA += acc;
-        }
-        hn = (x > 0.f) ? x : 0.f;
-        a.Hn[gi] = hn;
-      } else {
-        hn = h;
+  }
+  if (p2 >= 0) {
+    float hg[RP][4], qv[RP][4];
+#pragma unroll
+    for (int i = 0; i < RP; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) qv[i][j] = 0.f;
+    if (a.ncols2 > 0) parts_of<KP>(a.Q, a.nsplit2, a.skG2, a.ncols2, a.n2, p2, rg, cg, qv);
+    rows_times<KP>(Hs, G2, rg, cg, hg);
+#pragma unroll
+    for (int i = 0; i < RP; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float q = has3 ? rv[i][j] + qv[i][j] : qv[i][j];
+        g[i][j] = fmaf(a.coef, hg[i][j] - q, g[i][j]);
       }
+  }
+  if (p1 < 0 && p2 < 0) {
+#pragma unroll
+    for (int i = 0; i < RP; ++i) {
+      const float4 v = ld4(a.mu, i);
+      g[i][0] = v.x;
+      g[i][1] = v.y;
+      g[i][2] = v.z;
+      g[i][3] = v.w;
     }
-    Hn[r][c] = hn;
+  }
+  // outputs of the gradient
+#pragma unroll
+  for (int i = 0; i < RP; ++i) {
+    const bool in = rg + i * RS < rows;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (!in || c0 + j >= a.k) g[i][j] = 0.f;
+      const float pg = (h[i][j] > 0.f) ? g[i][j] : fminf(0.f, g[i][j]);
+      kkt2 = fmaf(pg, pg, kkt2);
+      if (!isfinite(g[i][j])) ++nonfin;
+      if (a.gcaller && in && c0 + j < a.k)
+        a.gcaller[(r0 + rg + i * RS) * a.k + c0 + j] = g[i][j];
+    }
+    if (a.gout) st4(a.gout, i, g[i]);
+    if (a.store_mu) st4(a.mu, i, g[i]);
+  }
+  if (a.update) {
+    __syncthreads();  // every thread has read H_t from Hs
+    float xv[RP][4];
+    if (admm) {
+      // H = rhs (2 W^T W + rho I)^-1 with rhs = 2 (S W) + rho (W - U), W' =
+      // [H + U]_+, U' = U + H - W' (appendix, Family 6)
+#pragma unroll
+      for (int i = 0; i < RP; ++i) {
+        const float4 u = ld4(a.A, i);
+        const float u4[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          Hs[rg + i * RS][c0 + j] = (rg + i * RS < rows && c0 + j < a.k)
+                                        ? fmaf(a.rho, h[i][j] - u4[j], 2.f * pv[i][j])
+                                        : 0.f;
+      }
+      for (int e = tid; e < KP * KP / 4; e += T)
+        reinterpret_cast<float4 *>(G1)[e] = reinterpret_cast<const float4 *>(a.minv)[e];
+      __syncthreads();
+      rows_times<KP>(Hs, G1, rg, cg, xv);
+      __syncthreads();  // every thread has read the right-hand sides
+    }
+#pragma unroll
+    for (int i = 0; i < RP; ++i) {
+      const float4 av4 = ld4(a.A, i);
+      const float4 mv4 = rms ? ld4(a.M, i) : make_float4(0.f, 0.f, 0.f, 0.f);
+      float av[4] = {av4.x, av4.y, av4.z, av4.w}, mv[4] = {mv4.x, mv4.y, mv4.z, mv4.w}, hn[4];
+      const bool in = rg + i * RS < rows;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        hn[j] = 0.f;
+        if (in && c0 + j < a.k) {
+          const float gv = g[i][j];
+          float x;
+          if (admm) {
+            x = xv[i][j] + av[j];
+            hn[j] = (x > 0.f) ? x : 0.f;
+            av[j] = x - hn[j];
+            sumA += av[j];
+          } else {
+            if (rms) {
+              av[j] = fmaf(a.alpha, av[j], __fmul_rn(1.f - a.alpha, __fmul_rn(gv, gv)));
+              mv[j] = fmaf(a.mom, mv[j], adaptive_step(a.eta * gv, av[j], a.eps));
+              x = h[i][j] - mv[j];
+            } else {
+              av[j] = fmaf(gv, gv, av[j]);
+              x = __fsub_rn(h[i][j], adaptive_step(a.eta * gv, av[j], a.eps));
+            }
+            sumA += av[j];
+            hn[j] = (x > 0.f) ? x : 0.f;
+          }
+        }
+        Hs[rg + i * RS][c0 + j] = hn[j];
+      }
+      st4(a.A, i, av);
+      if (rms) st4(a.M, i, mv);
+      st4(a.Hn, i, hn);
+    }
+    __syncthreads();  // Hs holds the tile of H_{t+1}
+    tile_tail<KP, T>(Hs, r0, a.Btn, a.bt_fmt, a.ldb, a.gram_part, tile);
+  }
+  // tile scalars: warp xor trees in float-float form, warps in order in FP64
+  float fh[3] = {tr, kkt2, sumA}, fl[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) ff_xor_add(fh[i], fl[i], o);
+  const unsigned nf = __reduce_add_sync(0xffffffffu, (unsigned)nonfin);
+  if ((tid & 31) == 0) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) red[tid >> 5][i] = (double)fh[i] + (double)fl[i];
+    red[tid >> 5][3] = (double)nf;
   }
   __syncthreads();
-  if (a.update && admm) {
-    // H = rhs (2 W^T W + rho I)^-1, W' = [H + U]_+, U' = U + H - W'
-    // (appendix, Family 6)
-    float xv[EPT];
+  if (tid < 4 && a.slots) {
+    double s = 0.0;
 #pragma unroll
-    for (int i = 0; i < EPT; ++i) {
-      const int e = tid + i * kEpiThreads;
-      const int r = e / KP, c = e % KP;
-      float x = 0.f;
-      if (r < rows && c < a.k) {
-#pragma unroll 8
-        for (int d = 0; d < KP; ++d) x = fmaf(Hn[r][d], a.minv[d * KP + c], x);
-        x += av[i];
-      }
-      xv[i] = x;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < EPT; ++i) {
-      const int e = tid + i * kEpiThreads;
-      const int r = e / KP, c = e % KP;
-      float w = 0.f;
-      if (r < rows && c < a.k) {
-        const int64_t gi = (r0 + r) * KP + c;
-        w = (xv[i] > 0.f) ? xv[i] : 0.f;
-        const float u = xv[i] - w;
-        a.A[gi] = u;
-        a.Hn[gi] = w;
-        sumA += u;
-      }
-      Hn[r][c] = w;
-    }
-    __syncthreads();
+    for (int w = 0; w < T / 32; ++w) s += red[w][tid];
+    a.slots[(int64_t)tile * kSlotStride + tid] = s;
   }
-  if (a.update) tile_tail<KP>(Hn, r0, a.Btn, a.bt_fmt, a.ldb, a.gram_part, tile);
-  const double s_tr = block_sum((double)tr, red);
-  const double s_kkt = block_sum((double)kkt2, red);
-  const double s_a = block_sum((double)sumA, red);
-  const double s_nf = block_sum((double)nonfin, red);
-  if (tid == 0 && a.slots) {
-    double *sl = a.slots + (int64_t)tile * kSlotStride;
-    sl[0] = s_tr;
-    sl[1] = s_kkt;
-    sl[2] = s_a;
-    sl[3] = s_nf;
-  }
-
-
 }
 
 template <int KP>
@@ -310,7 +430,7 @@ __global__ void __launch_bounds__(256) prepare_kernel(const float *H, int64_t n,
     Hn[r][c] = (r < rows) ? H[(r0 + r) * KP + c] : 0.f;
   }
   __syncthreads();
-  tile_tail<KP>(Hn, r0, Bt, bt_fmt, ldb, gram_part, tile);
+  tile_tail<KP, 256>(Hn, r0, Bt, bt_fmt, ldb, gram_part, tile);
 }
 
 // Fixed-order FP64 reduction of an iteration's per-tile results (the 4
@@ -604,11 +724,11 @@ __global__ void __launch_bounds__(256) admm_minv_kernel(const double *gram64, in
 
 cudaError_t launch_epilogue(const EpiArgs &a, cudaStream_t s) {
   KP_SWITCH(a.kp, {
-    constexpr size_t bytes = epi_smem_bytes<KPV>();
+    constexpr size_t bytes = EpiK<KPV>::SMEM;
     cudaError_t e = cudaFuncSetAttribute(epilogue_kernel<KPV>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
-    epilogue_kernel<KPV><<<a.ntiles, kEpiThreads, bytes, s>>>(a);
+    epilogue_kernel<KPV><<<a.ntiles, EpiK<KPV>::T, bytes, s>>>(a);
   });
   return cudaGetLastError();
 }

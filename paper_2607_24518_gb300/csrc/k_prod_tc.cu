@@ -571,16 +571,16 @@ __device__ __forceinline__ void tile_finish(const EpiArgs &e, int tp, float (&p)
               av[s] = x - ((x > 0.f) ? x : 0.f);
               sumA += av[s];
             } else if (rms) {
-              const float v = e.alpha * av[s] + (1.f - e.alpha) * (g * g);
+              const float v = fmaf(e.alpha, av[s], __fmul_rn(1.f - e.alpha, __fmul_rn(g, g)));
               av[s] = v;
-              const float m = e.mom * mv[s] + adaptive_step(e.eta * g, v, e.eps);
+              const float m = fmaf(e.mom, mv[s], adaptive_step(e.eta * g, v, e.eps));
               mv[s] = m;
               x = h - m;
               sumA += v;
             } else {
-              const float acc = av[s] + g * g;
+              const float acc = fmaf(g, g, av[s]);
               av[s] = acc;
-              x = h - adaptive_step(e.eta * g, acc, e.eps);
+              x = __fsub_rn(h, adaptive_step(e.eta * g, acc, e.eps));
               sumA += acc;
             }
             hn[j] = (x > 0.f) ? x : 0.f;
