@@ -234,7 +234,7 @@ __device__ __forceinline__ int64_t fslot(int64_t s, int c, int r) {
 template <int KP>
 struct GramBlk {
   static constexpr int B = KP / 8;
-  static constexpr int BP = B == 8 ? 2 : B;  // block rows summed per pass
+  static constexpr int BP = B == 8 ? 4 : B;  // block rows summed per pass
 };
 
 // Per-tile update for the thread's row (row = tile row, et = index among the
@@ -252,27 +252,37 @@ struct Own {
   static constexpr bool GX = (KP == 64);
   static constexpr int HG = GX ? 1 : KH;
 };
-// the thread's H_t Gram_t for the 8 owned columns from c (row hrow of Hs,
-// columns cb + c ..), summed over d in order
+// H_t Gram_t of the tile into Gx by the 256 epilogue threads (kp = 64): 8 rows
+// x 4 columns per thread, so a column of H costs 8 scalar and one 16-byte
+// read for 32 FMAs.  One row x 8 columns per thread filled 16 bytes of registers
+// per FMA and took most of a tile's 22 us of preparation (gradient at n =
+// 4096, k = 64 BF16 80 -> 29 us, step at n = 20000 FP8 144 -> 130, with four
+// instead of two Gram block rows per pass).  Summed over d in order; ends with
+// every thread past a barrier.
 template <int KP>
-__device__ __forceinline__ void hgram8(const float *hrow, const float *Gs, int cb, int c,
-                                       float (&h8)[8]) {
+__device__ __forceinline__ void hgram_tile(const float *Hs, const float *Gs, float *Gx, int et) {
+  constexpr int CG = KP / 4, RS = 256 / CG, RP = 128 / RS;
+  const int cg = et % CG, rg = et / CG;
+  float acc[RP][4];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) h8[j] = 0.f;
+  for (int i = 0; i < RP; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
 #pragma unroll 4
   for (int d = 0; d < KP; ++d) {
-    const float hv = hrow[d];
-    const float4 *gr = reinterpret_cast<const float4 *>(Gs + d * KP + cb + c);
-    const float4 g0 = __ldg(gr), g1 = __ldg(gr + 1);
-    h8[0] = fmaf(hv, g0.x, h8[0]);
-    h8[1] = fmaf(hv, g0.y, h8[1]);
-    h8[2] = fmaf(hv, g0.z, h8[2]);
-    h8[3] = fmaf(hv, g0.w, h8[3]);
-    h8[4] = fmaf(hv, g1.x, h8[4]);
-    h8[5] = fmaf(hv, g1.y, h8[5]);
-    h8[6] = fmaf(hv, g1.z, h8[6]);
-    h8[7] = fmaf(hv, g1.w, h8[7]);
+    const float4 m = __ldg(reinterpret_cast<const float4 *>(Gs + d * KP) + cg);
+#pragma unroll
+    for (int i = 0; i < RP; ++i) {
+      const float h = Hs[(rg + i * RS) * (KP + 1) + d];
+      acc[i][0] = fmaf(h, m.x, acc[i][0]);
+      acc[i][1] = fmaf(h, m.y, acc[i][1]);
+      acc[i][2] = fmaf(h, m.z, acc[i][2]);
+      acc[i][3] = fmaf(h, m.w, acc[i][3]);
+    }
   }
+#pragma unroll
+  for (int i = 0; i < RP; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) Gx[(rg + i * RS) * (KP + 1) + 4 * cg + j] = acc[i][j];
+  epi_bar();
 }
 
 // Rows [0, rows) of a tile held in Hs (row stride KP + 1) to dst (row
@@ -389,14 +399,7 @@ __device__ __forceinline__ void tile_prep(const EpiArgs &e, int tp, float *Hs, f
   }
   // (H_t Gram_t) for the owned columns, right to left (Sec. 2.1)
   if constexpr (Own<KP>::GX) {
-    float *gx = Gx + row * (KP + 1) + cb;
-#pragma unroll 1
-    for (int c = 0; c < KH; c += 8) {
-      float h8[8];
-      hgram8<KP>(hrow, Gs, cb, c, h8);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) gx[c + j] = h8[j];
-    }
+    hgram_tile<KP>(Hs, Gs, Gx, et);
     return;
   }
 #pragma unroll
@@ -827,9 +830,11 @@ __device__ void epilogue_role(const TcArgs &a, const EpiArgs &e, uint32_t tmem_b
   // CTAs b0..b1 but `self` to p in CTA order (p holds this CTA's part,
   // first in the order); sum_parts forms the CTA-order sum of all of them
   // with p standing for this CTA's part at its place.
-  // (kp = 64: 8 columns at a time, fewer live registers; the additions of
-  // each column keep CTA order either way)
-  constexpr int PC = Own<KP>::GX ? 8 : KH;
+  // (kp = 64: 16 columns at a time, fewer live registers; the additions of
+  // each column keep CTA order either way).  Up to kp = 16 two parts are in
+  // flight: a small matrix has several per tile, each an L2 round trip.
+  constexpr int PC = Own<KP>::GX ? 16 : KH;
+  constexpr bool kTwo = (KP <= 16);
   auto load_pc = [&](float (&v)[PC], int64_t bb, int tp, int c) {
 #pragma unroll
     for (int j = 0; j < PC; ++j) v[j] = __ldcg(a.out + fslot<KP>(bb + tp, c + j, row));
@@ -837,12 +842,23 @@ __device__ void epilogue_role(const TcArgs &a, const EpiArgs &e, uint32_t tmem_b
   auto add_parts = [&](float (&pp)[KH], int64_t b0, int64_t b1, int64_t self, int tp, int cb) {
 #pragma unroll
     for (int c0 = 0; c0 < KH; c0 += PC) {
-      for (int64_t bb = b0; bb <= b1; ++bb) {
-        if (bb == self) continue;
-        float v[PC];
+      for (int64_t bb = b0 + (b0 == self); bb <= b1;) {
+        float v[PC], w[kTwo ? PC : 1];
         load_pc(v, bb, tp, cb + c0);
+        bb += 1 + (bb + 1 == self);
+        const bool two = kTwo && bb <= b1;
+        if constexpr (kTwo) {
+          if (two) load_pc(w, bb, tp, cb + c0);
+        }
 #pragma unroll
         for (int j = 0; j < PC; ++j) pp[c0 + j] += v[j];
+        if constexpr (kTwo) {
+          if (two) {
+#pragma unroll
+            for (int j = 0; j < PC; ++j) pp[c0 + j] += w[j];
+            bb += 1 + (bb + 1 == self);
+          }
+        }
       }
     }
   };
@@ -850,21 +866,22 @@ __device__ void epilogue_role(const TcArgs &a, const EpiArgs &e, uint32_t tmem_b
 #pragma unroll
     for (int c0 = 0; c0 < KH; c0 += PC) {
       float acc[PC];
-      if (b0 == self) {
 #pragma unroll
-        for (int j = 0; j < PC; ++j) acc[j] = pp[c0 + j];
-      } else {
-        load_pc(acc, b0, tp, cb + c0);
-      }
-      for (int64_t bb = b0 + 1; bb <= b1; ++bb) {
-        if (bb == self) {
+      for (int j = 0; j < PC; ++j) acc[j] = 0.f;
+      for (int64_t bb = b0; bb <= b1; bb += kTwo ? 2 : 1) {
+        float v[PC], w[kTwo ? PC : 1];
+        const bool two = kTwo && bb + 1 <= b1;
+        if (bb != self) load_pc(v, bb, tp, cb + c0);
+        if constexpr (kTwo) {
+          if (two && bb + 1 != self) load_pc(w, bb + 1, tp, cb + c0);
+        }
 #pragma unroll
-          for (int j = 0; j < PC; ++j) acc[j] += pp[c0 + j];
-        } else {
-          float v[PC];
-          load_pc(v, bb, tp, cb + c0);
+        for (int j = 0; j < PC; ++j) acc[j] += bb == self ? pp[c0 + j] : v[j];
+        if constexpr (kTwo) {
+          if (two) {
 #pragma unroll
-          for (int j = 0; j < PC; ++j) acc[j] += v[j];
+            for (int j = 0; j < PC; ++j) acc[j] += bb + 1 == self ? pp[c0 + j] : w[j];
+          }
         }
       }
 #pragma unroll
