@@ -1565,6 +1565,13 @@ __global__ void __launch_bounds__(Cfg<DT, KP>::THREADS, 1)
       int stage = 0;
       uint32_t phase = 0;
       bool stop = false;
+      // S passes through L2 first to go: with the default policy its stream
+      // evicts the state, the factor and its MMA copy in every iteration, and
+      // the tile epilogues' loads then queue behind it for HBM (8 to 10 us a
+      // round trip).  n = 20000: FP32 k = 32 273 -> 268 us, BF16 138 -> 130
+      // (k = 64 198 -> 167), FP8 87 -> 82 (131 -> 118); a matrix that fits L2
+      // stays in it either way.
+      const uint64_t pol = l2_evict_first();
       for (int si = 0; si < 2 && !stop; ++si) {
         if (sg.hi[si] <= sg.lo[si]) continue;
         int tp = (int)(sg.lo[si] / a.n_cols);
@@ -1587,7 +1594,8 @@ __global__ void __launch_bounds__(Cfg<DT, KP>::THREADS, 1)
             mbar_expect_tx(&full[stage], C::STAGE);
 #pragma unroll
             for (int at = 0; at < C::APS; ++at) {
-              tma_load_2d(sa + at * kAtomBytes, &mapS, &full[stage], x0 + at * C::ATOM_COLS, rt * 128);
+              tma_load_2d_hint(sa + at * kAtomBytes, &mapS, &full[stage], x0 + at * C::ATOM_COLS,
+                               rt * 128, pol);
               tma_load_2d(sb + at * C::B_ATOM, &mapB, &full[stage], x0 + at * C::ATOM_COLS, 0);
             }
             if constexpr (C::SLO16)  // bf16 H^T rows for the stage's 64 columns
