@@ -1735,6 +1735,20 @@ cudaError_t launch_step_tc(const ProdArgs &a, const EpiArgs *epi, int *tile_cnt,
   TcArgs ta{};
   ta.W = (int64_t)a.n_rows_list * a.n_cols_list;
   ta.G = (int)std::max<int64_t>(1, std::min<int64_t>(ta.W, num_sms));
+  // A grid of m CTAs per row tile shares no CTA between two tiles (b W / G is
+  // then a tile boundary for every m-th b), so no CTA has to finish two tiles
+  // one after the other: an epilogue is 10 us, 20 at kp = 64.  Taken while the
+  // fuller shares cost less than that; a unit takes 0.5 (FP8) to 2 us (FP32; 4
+  // at kp = 64).  n = 4000: BF16 k = 8 / 32 / 64 24.5 / 46 / 87 -> 15.4 / 25 /
+  // 40 us, FP8 25 / 44 / 80 -> 16 / 26 / 44, FP32 k = 32 37 -> 31; n = 8000,
+  // k = 32: BF16 the same (36), FP8 41 -> 30; beyond the limits it loses (FP32
+  // n = 8000, 32 instead of 27 units: k = 16 56 -> 59, k = 64 131 -> 147).
+  if (epi && a.n_rows_list < num_sms) {
+    const int m = std::min(num_sms / a.n_rows_list, a.n_cols_list);
+    const int whole = (a.n_cols_list + m - 1) / m, share = (int)((ta.W + ta.G - 1) / ta.G);
+    const int most = a.dtype == 0 ? (a.kp == 64 ? 0 : 3) : a.kp == 64 ? 3 : 8;
+    if (whole - share <= most) ta.G = m * a.n_rows_list;
+  }
   ta.n_cols = a.n_cols_list;
   ta.row_list = a.row_list;
   ta.col_list = a.col_list;
