@@ -47,7 +47,9 @@ struct symnmf_ctx {
   int num_sms = 0;
   int impl_req = 0;   // 0 auto, 1 simt, 2 tc
   bool tc_layout_ok = false;
-  // owned device memory
+  // owned device memory: one block, and one pinned block on the host, that
+  // the pointers below divide (carve_device, carve_host)
+  uint8_t *arena = nullptr, *harena = nullptr;
   float *H[2] = {nullptr, nullptr};
   void *Bt[2] = {nullptr, nullptr};
   int bt_fmt = 0;          // 0: bf16 hi/lo, 1: tf32 hi/lo in float, 2: e4m3 pieces
@@ -56,10 +58,10 @@ struct symnmf_ctx {
   float *gram32[2] = {nullptr, nullptr};
   int cur = 0;
   float *A = nullptr, *M = nullptr, *mu = nullptr, *g = nullptr, *tmp = nullptr;
-  float *P = nullptr, *Q = nullptr, *R = nullptr;  // product partials
+  float *P = nullptr, *Q = nullptr, *R = nullptr;  // product partials, one after the other
+  size_t pqr_bytes = 0;
   int64_t pq_cap_tiles = 0;
-  double *slots = nullptr, *chunk = nullptr;
-  int nchunks = 1;
+  double *slots = nullptr;
   float *gramI = nullptr, *gramJ = nullptr;
   float *minv = nullptr;    // ADMM: (2 Gram_t + rho I)^-1
   int *dlists = nullptr;    // kStages x kListArrays x ntiles
@@ -155,25 +157,64 @@ cudaError_t dalloc(T **p, size_t count) {
   return e;
 }
 
-void free_all(symnmf_t h) {
-  for (int i = 0; i < 2; ++i) {
-    cudaFree(h->H[i]);
-    cudaFree(h->Bt[i]);
-    cudaFree(h->gram_part[i]);
-    cudaFree(h->gram64[i]);
-    cudaFree(h->gram32[i]);
+// Sub-allocation of one block: take() hands out 256-byte aligned ranges; with
+// a null base it only adds up the size.
+struct Carve {
+  uint8_t *base;
+  size_t used = 0;
+  template <class T>
+  void take(T **p, size_t count) {
+    *p = base ? reinterpret_cast<T *>(base + used) : nullptr;
+    used += (std::max<size_t>(1, count) * sizeof(T) + 255) & ~(size_t)255;
   }
-  for (void *p : {(void *)h->A, (void *)h->M, (void *)h->mu, (void *)h->g, (void *)h->tmp,
-                  (void *)h->P, (void *)h->Q, (void *)h->R, (void *)h->slots, (void *)h->chunk,
-                  (void *)h->gramI, (void *)h->gramJ, (void *)h->minv, (void *)h->dlists, (void *)h->ring,
-                  (void *)h->hist, (void *)h->sel, (void *)h->dmed, (void *)h->dsum,
-                  (void *)h->norm_parts, (void *)h->dev_err, (void *)h->tile_cnt,
-                  (void *)h->km_rn, (void *)h->km_lab, (void *)h->km_colsq,
+};
+
+size_t carve_device(symnmf_t h, uint8_t *base) {
+  Carve c{base};
+  const size_t nkp = (size_t)h->ntiles * kTileRows * h->kp, kk = (size_t)h->kp * h->kp;
+  for (int i = 0; i < 2; ++i) {
+    c.take(&h->H[i], nkp);
+    c.take(reinterpret_cast<uint8_t **>(&h->Bt[i]), bt_bytes(h->bt_fmt, h->kp, h->ldb));
+    c.take(&h->gram_part[i], h->ntiles * kk);
+    c.take(&h->gram64[i], kk);
+    c.take(&h->gram32[i], kk);
+  }
+  for (float **p : {&h->A, &h->M, &h->mu, &h->g, &h->tmp}) c.take(p, nkp);
+  const size_t pqr0 = c.used;
+  for (float **p : {&h->P, &h->Q, &h->R}) c.take(p, (size_t)h->pq_cap_tiles * kTileRows * h->kp);
+  h->pqr_bytes = c.used - pqr0;
+  c.take(&h->slots, (size_t)h->ntiles * kSlotStride);
+  c.take(&h->gramI, kk);
+  c.take(&h->gramJ, kk);
+  c.take(&h->minv, kk);
+  c.take(&h->dlists, (size_t)kStages * kListArrays * h->ntiles);
+  c.take(&h->ring, (size_t)kRing + 1);
+  c.take(&h->hist, 2048);
+  c.take(&h->sel, 4);
+  c.take(&h->dmed, 1);
+  c.take(&h->dsum, 4);
+  c.take(&h->norm_parts, (size_t)h->n_norm_parts);
+  c.take(&h->dev_err, 4);
+  c.take(&h->tile_cnt, (size_t)h->ntiles);
+  return c.used;
+}
+
+size_t carve_host(symnmf_t h, uint8_t *base) {
+  Carve c{base};
+  c.take(&h->host_err, 4);
+  c.take(&h->hlists, (size_t)kStages * kListArrays * h->ntiles);
+  c.take(&h->hring, (size_t)kRing + 1);
+  c.take(&h->hsum, 4);
+  c.take(&h->hmed, 4);
+  return c.used;
+}
+
+void free_all(symnmf_t h) {
+  for (void *p : {(void *)h->arena, (void *)h->km_rn, (void *)h->km_lab, (void *)h->km_colsq,
                   (void *)h->km_inv, (void *)h->km_slots, (void *)h->km_out, (void *)h->rs_part,
                   (void *)h->rs_out})
-    cudaFree(p);
-  for (void *p : {(void *)h->hlists, (void *)h->hring, (void *)h->hsum, (void *)h->hmed,
-                  (void *)h->host_err, (void *)h->km_hout, (void *)h->rs_host})
+    if (p) cudaFree(p);
+  for (void *p : {(void *)h->harena, (void *)h->km_hout, (void *)h->rs_host})
     if (p) cudaFreeHost(p);
   for (int i = 0; i < kStages; ++i)
     if (h->stage_ev[i]) cudaEventDestroy(h->stage_ev[i]);
@@ -928,45 +969,18 @@ int symnmf_create_ld(const void *S, int64_t n, int64_t lds, int32_t k, int32_t d
   reset_ctrl(&h->ctrl);
   cudaError_t e = cudaGetDevice(&h->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
-  const int64_t nkp = (int64_t)h->ntiles * kTileRows * h->kp;  // tile column-major
   h->pq_cap_tiles = h->ntiles + 3 * (int64_t)std::max(1, h->num_sms);
-  h->nchunks = std::max(1, std::min(h->ntiles, 64));
   h->n_norm_parts = 4 * std::max(1, h->num_sms);
-  for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
-    e = dalloc(&h->H[i], nkp);
-    if (e == cudaSuccess)
-      e = dalloc((uint8_t **)&h->Bt[i], bt_bytes(h->bt_fmt, h->kp, h->ldb));
-    if (e == cudaSuccess) e = dalloc(&h->gram_part[i], (size_t)h->ntiles * h->kp * h->kp);
-    if (e == cudaSuccess) e = dalloc(&h->gram64[i], (size_t)h->kp * h->kp);
-    if (e == cudaSuccess) e = dalloc(&h->gram32[i], (size_t)h->kp * h->kp);
+  // one device block and one pinned block: 32 allocations, each zeroed on its
+  // own, and as many frees took about 0.7 ms of a handle's life
+  const size_t bytes = carve_device(h, nullptr);
+  if (e == cudaSuccess) e = cudaMalloc((void **)&h->arena, bytes);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->arena, 0, bytes, nullptr);
+  if (e == cudaSuccess) e = cudaMallocHost((void **)&h->harena, carve_host(h, nullptr));
+  if (e == cudaSuccess) {
+    carve_device(h, h->arena);
+    carve_host(h, h->harena);
   }
-  if (e == cudaSuccess) e = dalloc(&h->A, nkp);
-  if (e == cudaSuccess) e = dalloc(&h->M, nkp);
-  if (e == cudaSuccess) e = dalloc(&h->mu, nkp);
-  if (e == cudaSuccess) e = dalloc(&h->g, nkp);
-  if (e == cudaSuccess) e = dalloc(&h->tmp, nkp);
-  if (e == cudaSuccess) e = dalloc(&h->P, (size_t)h->pq_cap_tiles * kTileRows * h->kp);
-  if (e == cudaSuccess) e = dalloc(&h->Q, (size_t)h->pq_cap_tiles * kTileRows * h->kp);
-  if (e == cudaSuccess) e = dalloc(&h->R, (size_t)h->pq_cap_tiles * kTileRows * h->kp);
-  if (e == cudaSuccess) e = dalloc(&h->slots, (size_t)h->ntiles * kSlotStride);
-  if (e == cudaSuccess) e = dalloc(&h->chunk, (size_t)h->nchunks * (4 + h->kp * h->kp));
-  if (e == cudaSuccess) e = dalloc(&h->gramI, (size_t)h->kp * h->kp);
-  if (e == cudaSuccess) e = dalloc(&h->gramJ, (size_t)h->kp * h->kp);
-  if (e == cudaSuccess) e = dalloc(&h->minv, (size_t)h->kp * h->kp);
-  if (e == cudaSuccess) e = dalloc(&h->dlists, (size_t)kStages * kListArrays * h->ntiles);
-  if (e == cudaSuccess) e = dalloc(&h->ring, (size_t)kRing + 1);
-  if (e == cudaSuccess) e = dalloc(&h->hist, 2048);
-  if (e == cudaSuccess) e = dalloc(&h->sel, 4);
-  if (e == cudaSuccess) e = dalloc(&h->dmed, 1);
-  if (e == cudaSuccess) e = dalloc(&h->dsum, 4);
-  if (e == cudaSuccess) e = dalloc(&h->norm_parts, (size_t)h->n_norm_parts);
-  if (e == cudaSuccess) e = dalloc(&h->dev_err, 4);
-  if (e == cudaSuccess) e = dalloc(&h->tile_cnt, (size_t)h->ntiles);
-  if (e == cudaSuccess) e = cudaMallocHost((void **)&h->host_err, sizeof(int) * 4);
-  if (e == cudaSuccess) e = cudaMallocHost((void **)&h->hlists, sizeof(int) * kStages * kListArrays * h->ntiles);
-  if (e == cudaSuccess) e = cudaMallocHost((void **)&h->hring, sizeof(DevRecord) * (kRing + 1));
-  if (e == cudaSuccess) e = cudaMallocHost((void **)&h->hsum, sizeof(double) * 4);
-  if (e == cudaSuccess) e = cudaMallocHost((void **)&h->hmed, sizeof(float) * 4);
   for (int i = 0; i < kStages && e == cudaSuccess; ++i)
     e = cudaEventCreateWithFlags(&h->stage_ev[i], cudaEventDisableTiming);
   if (e != cudaSuccess) {
@@ -983,6 +997,11 @@ int symnmf_create_ld(const void *S, int64_t n, int64_t lds, int32_t k, int32_t d
       delete h;
       return rc;
     }
+  } else if (cudaStreamSynchronize(nullptr) != cudaSuccess) {
+    // (the block is zero before any stream of the caller's touches it)
+    free_all(h);
+    delete h;
+    return SYMNMF_ERR_CUDA;
   }
   *out = h;
   return SYMNMF_OK;
@@ -1105,19 +1124,18 @@ int symnmf_window_update(symnmf_t h, const float *Y, int64_t T, int64_t ldy, int
   const bool f8 = (h->dtype == SYMNMF_FP8E4M3);
   if (f8 && (!scales || ld_scales < h->ntiles)) return SYMNMF_ERR_INVALID;
   if (h->n > 2097120 || T > (int64_t)1 << 30) return SYMNMF_ERR_UNSUPPORTED;
-  CK(cudaMemsetAsync(h->dev_err, 0, sizeof(int), h->stream));
   // the build, ordered after every launch that reads the old matrix; it
-  // leaves ||S||^2 of the stored values in dsum (F32 / BF16)
+  // leaves ||S||^2 of the stored values in dsum (F32 / BF16).  The partial
+  // slots, which hold nothing between iterations, are its workspace
   const int dt = h->dtype == SYMNMF_F32 ? 0 : h->dtype == SYMNMF_BF16 ? 1 : 2;
   cudaError_t e = launch_dependence(Y, T, h->n, ldy, center ? 1 : 0, dt, S, lds, scales,
-                                    ld_scales, f8 ? nullptr : h->dsum, h->dev_err, h->stream,
-                                    true);
+                                    ld_scales, f8 ? nullptr : h->dsum, h->dev_err, h->host_err,
+                                    h->stream, true, h->P, h->pqr_bytes);
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
     return fail(h, SYMNMF_ERR_OOM, "dependence build scratch");
   }
   if (e != cudaSuccess) return cuda_fail(h, e, "dependence build");
-  CK(cudaMemcpyAsync(h->host_err, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   int rc = rebind_matrix(h, S, lds, scales, ld_scales);
   if (rc) return rc;
   if (f8) {
@@ -1366,20 +1384,10 @@ int symnmf_build_dependence(const float *Y, int64_t T, int64_t n, int64_t ldy, i
   if (out_dtype == SYMNMF_FP8E4M3 && (!scales || ld_scales < nt)) return SYMNMF_ERR_INVALID;
   if (n > 2097120 || T > (int64_t)1 << 30) return SYMNMF_ERR_UNSUPPORTED;
   cudaStream_t s = (cudaStream_t)stream;
-  int *derr = nullptr;
   int herr = 0;
-  cudaError_t e = cudaMallocAsync((void **)&derr, sizeof(int), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(derr, 0, sizeof(int), s);
-  if (e == cudaSuccess) {
-    const int dt = out_dtype == SYMNMF_F32 ? 0 : out_dtype == SYMNMF_BF16 ? 1 : 2;
-    e = launch_dependence(Y, T, n, ldy, center ? 1 : 0, dt, S, lds, scales, ld_scales, normS2,
-                          derr, s);
-  }
-  if (derr) {
-    cudaError_t e2 = cudaMemcpyAsync(&herr, derr, sizeof(int), cudaMemcpyDeviceToHost, s);
-    cudaFreeAsync(derr, s);
-    if (e == cudaSuccess) e = e2;
-  }
+  const int dt = out_dtype == SYMNMF_F32 ? 0 : out_dtype == SYMNMF_BF16 ? 1 : 2;
+  cudaError_t e = launch_dependence(Y, T, n, ldy, center ? 1 : 0, dt, S, lds, scales, ld_scales,
+                                    normS2, nullptr, &herr, s);
   cudaError_t es2 = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = es2;
   if (e == cudaErrorMemoryAllocation) {

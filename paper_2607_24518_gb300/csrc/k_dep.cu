@@ -620,7 +620,8 @@ __global__ void __launch_bounds__(256) dep_sum_kernel(const double *x, int64_t m
 
 cudaError_t launch_dependence(const float *Y, int64_t T, int64_t n, int64_t ldy, int center,
                               int out, void *S, int64_t lds, float *scales, int64_t ld_scales,
-                              double *normS2, int *err, cudaStream_t s, bool exact_norm) {
+                              double *normS2, int *err, int *herr, cudaStream_t s,
+                              bool exact_norm, void *ws, size_t ws_bytes) {
   const int Tp = (int)((T + 31) / 32 * 32);
   const int nib = (int)((n + 127) / 128), njb = (int)((n + 255) / 256);
   if (nib >= 65536 || njb >= 65536) return cudaErrorInvalidValue;
@@ -632,21 +633,30 @@ cudaError_t launch_dependence(const float *Y, int64_t T, int64_t n, int64_t ldy,
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   const int G = std::max(1, std::min(sms, ntiles));
-  // one scratch block: P, then the CTA sums, then 1 / (s_i sqrt(d_i))
+  // one scratch block: P, then the CTA sums, the error word and 1 / (s_i sqrt(d_i))
   const size_t bytesP = sizeof(__half) * (size_t)n * 2 * Tp;  // a multiple of 128
-  uint8_t *scratch = nullptr;
-  e = cudaMallocAsync((void **)&scratch, bytesP + sizeof(double) * G + sizeof(float) * (size_t)n, s);
-  if (e != cudaSuccess) return e;
+  const size_t bytes = bytesP + sizeof(double) * (G + 1) + sizeof(float) * (size_t)n;
+  // (stream-ordered memory goes back to the system at every synchronisation,
+  // so it is mapped anew by each call: about 150 us)
+  uint8_t *scratch = reinterpret_cast<uint8_t *>(ws);
+  const bool own = !ws || ws_bytes < bytes;
+  if (own) {
+    e = cudaMallocAsync((void **)&scratch, bytes, s);
+    if (e != cudaSuccess) return e;
+  }
   __half *P = reinterpret_cast<__half *>(scratch);
   double *sq = reinterpret_cast<double *>(scratch + bytesP);
-  float *inv_d = reinterpret_cast<float *>(sq + G);
+  if (!err) err = reinterpret_cast<int *>(sq + G);
+  float *inv_d = reinterpret_cast<float *>(sq + G + 1);
+  e = cudaMemsetAsync(err, 0, sizeof(int), s);
   dep_prep_kernel<<<(unsigned)((n + 31) / 32), dim3(32, kPrepY), 0, s>>>(Y, T, n, ldy, center, Tp,
                                                                          inv_d, P);
   CUtensorMap mP;
-  if (!make_map_2d(&mP, P, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, (uint64_t)2 * Tp, (uint64_t)n,
+  if (e == cudaSuccess &&
+      !make_map_2d(&mP, P, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, (uint64_t)2 * Tp, (uint64_t)n,
                    (uint64_t)2 * Tp * 2, kDepKC, 128, 64)) {
     e = cudaErrorInvalidValue;
-  } else {
+  } else if (e == cudaSuccess) {
     e = cudaFuncSetAttribute(dep_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kDepSmem);
   }
@@ -670,8 +680,9 @@ cudaError_t launch_dependence(const float *Y, int64_t T, int64_t n, int64_t ldy,
     dep_gemm_kernel<<<(unsigned)G, kDepThreads, kDepSmem, s>>>(mP, a);
     if (normS2) dep_sum_kernel<<<1, 256, 0, s>>>(sq, G, normS2);
     e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(herr, err, sizeof(int), cudaMemcpyDeviceToHost, s);
   }
-  const cudaError_t e2 = cudaFreeAsync(scratch, s);
+  const cudaError_t e2 = own ? cudaFreeAsync(scratch, s) : cudaSuccess;
   return e == cudaSuccess ? e2 : e;
 }
 

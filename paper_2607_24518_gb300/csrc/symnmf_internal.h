@@ -209,12 +209,14 @@ cudaError_t launch_quantize_fp8(const void *src, int src_dtype, int64_t rows, in
 cudaError_t launch_sum_slot(const double *slots, int ntiles, int which, double *out,
                             cudaStream_t s);
 
-// Dependence matrix S = |D^-1/2 Y^T Y D^-1/2| (Sec. 3), k_dep.cu; err is a
-// device int the kernels set on a bounded-wait timeout
+// Dependence matrix S = |D^-1/2 Y^T Y D^-1/2| (Sec. 3), k_dep.cu.  err: device
+// int (nullptr: one in the build's scratch) that is zeroed, set on a
+// bounded-wait timeout and copied to *herr (host) on the stream.  ws: a
+// caller's workspace (256-byte aligned), used when the build's scratch fits
 cudaError_t launch_dependence(const float *Y, int64_t T, int64_t n, int64_t ldy, int center,
                               int out, void *S, int64_t lds, float *scales, int64_t ld_scales,
-                              double *normS2, int *err, cudaStream_t s,
-                              bool exact_norm = false);
+                              double *normS2, int *err, int *herr, cudaStream_t s,
+                              bool exact_norm = false, void *ws = nullptr, size_t ws_bytes = 0);
 
 // Spherical K-means (Sec. 6): the kernels around the two product passes of
 // one Lloyd iteration (k_kmeans.cu)
