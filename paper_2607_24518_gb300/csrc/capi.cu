@@ -110,6 +110,7 @@ struct symnmf_ctx {
   double *rs_part = nullptr, *rs_out = nullptr, *rs_host = nullptr;  // host: pinned
   // spherical K-means scratch, allocated by the first symnmf_spkmeans
   double *km_rn = nullptr;      // ||s_i||
+  float *km_rinv = nullptr;     // 1 / ||s_i||
   int *km_lab = nullptr;        // two label buffers of n
   double *km_colsq = nullptr;   // ntiles x kp
   float *km_inv = nullptr;      // kp
@@ -210,8 +211,8 @@ size_t carve_host(symnmf_t h, uint8_t *base) {
 }
 
 void free_all(symnmf_t h) {
-  for (void *p : {(void *)h->arena, (void *)h->km_rn, (void *)h->km_lab, (void *)h->km_colsq,
-                  (void *)h->km_inv, (void *)h->km_slots, (void *)h->km_out, (void *)h->rs_part,
+  for (void *p : {(void *)h->arena, (void *)h->km_rn, (void *)h->km_rinv, (void *)h->km_lab,
+                  (void *)h->km_colsq, (void *)h->km_inv, (void *)h->km_slots, (void *)h->km_out, (void *)h->rs_part,
                   (void *)h->rs_out})
     if (p) cudaFree(p);
   for (void *p : {(void *)h->harena, (void *)h->km_hout, (void *)h->rs_host})
@@ -1099,7 +1100,7 @@ static int rebind_matrix(symnmf_t h, const void *S, int64_t lds, const float *sc
   std::memset(&h->last_check_rec, 0, sizeof(h->last_check_rec));
   if (h->km_rn) {
     CK(launch_row_norms(h->S, h->n, h->lds, h->dtype, h->scales, h->ld_scales, h->km_rn,
-                        h->stream));
+                        h->km_rinv, h->stream));
   }
   return SYMNMF_OK;
 }
@@ -1407,6 +1408,7 @@ int symnmf_spkmeans(symnmf_t h, const int32_t *labels0, int32_t *labels, int32_t
     return fail(h, SYMNMF_ERR_INVALID, "spkmeans: null labels, max_iter < 1 or tol < 0");
   if (!h->km_rn) {
     cudaError_t e = dalloc(&h->km_rn, (size_t)h->n);
+    if (e == cudaSuccess) e = dalloc(&h->km_rinv, (size_t)h->n);
     if (e == cudaSuccess) e = dalloc(&h->km_lab, (size_t)2 * h->n);
     if (e == cudaSuccess) e = dalloc(&h->km_colsq, (size_t)h->ntiles * h->kp);
     if (e == cudaSuccess) e = dalloc(&h->km_inv, (size_t)h->kp);
@@ -1415,11 +1417,12 @@ int symnmf_spkmeans(symnmf_t h, const int32_t *labels0, int32_t *labels, int32_t
     if (e == cudaSuccess) e = cudaMallocHost((void **)&h->km_hout, 2 * sizeof(double));
     if (e != cudaSuccess) {
       cudaGetLastError();
-      for (void *p : {(void *)h->km_rn, (void *)h->km_lab, (void *)h->km_colsq, (void *)h->km_inv,
-                      (void *)h->km_slots, (void *)h->km_out})
+      for (void *p : {(void *)h->km_rn, (void *)h->km_rinv, (void *)h->km_lab, (void *)h->km_colsq,
+                      (void *)h->km_inv, (void *)h->km_slots, (void *)h->km_out})
         cudaFree(p);
       if (h->km_hout) cudaFreeHost(h->km_hout);
       h->km_rn = nullptr;
+      h->km_rinv = nullptr;
       h->km_lab = nullptr;
       h->km_colsq = nullptr;
       h->km_inv = nullptr;
@@ -1429,7 +1432,7 @@ int symnmf_spkmeans(symnmf_t h, const int32_t *labels0, int32_t *labels, int32_t
       return fail(h, SYMNMF_ERR_OOM, "spkmeans scratch");
     }
     CK(launch_row_norms(h->S, h->n, h->lds, h->dtype, h->scales, h->ld_scales, h->km_rn,
-                        h->stream));
+                        h->km_rinv, h->stream));
     count_kernels(h, 1);
   }
   // the two product operands go through the solver's other H buffer and MMA
@@ -1440,8 +1443,6 @@ int symnmf_spkmeans(symnmf_t h, const int32_t *labels0, int32_t *labels, int32_t
     ~KeepCur() { h->cur = c; }
   } keep{h, h->cur};
   h->cur = 1 - keep.c;
-  float *Hop = h->H[h->cur];
-  const int64_t rows_alloc = (int64_t)h->ntiles * kTileRows;
   CK(cudaMemcpyAsync(h->km_lab, labels0, sizeof(int32_t) * h->n, cudaMemcpyDeviceToDevice,
                      h->stream));
   KmArgs a{};
@@ -1449,7 +1450,11 @@ int symnmf_spkmeans(symnmf_t h, const int32_t *labels0, int32_t *labels, int32_t
   a.K = h->k;
   a.ntiles = h->ntiles;
   a.P = h->P;
-  a.C = Hop;
+  a.C = use_tc(h) ? nullptr : h->H[h->cur];
+  a.Bt = h->Bt[h->cur];
+  a.bt_fmt = h->bt_fmt;
+  a.ldb = h->ldb;
+  a.rinv = h->km_rinv;
   a.colsq = h->km_colsq;
   a.inv_norm = h->km_inv;
   a.rn = h->km_rn;
@@ -1462,9 +1467,9 @@ int symnmf_spkmeans(symnmf_t h, const int32_t *labels0, int32_t *labels, int32_t
     int *lin = h->km_lab + (size_t)li * h->n;
     int *lout = h->km_lab + (size_t)(1 - li) * h->n;
     // pass 1: C = S (D^-1 B)
-    CK(launch_km_operand(lin, h->km_rn, h->n, h->kp, Hop, rows_alloc, h->stream));
-    CK(launch_prepare_tiles(Hop, h->n, h->k, h->kp, h->Bt[h->cur], h->bt_fmt, h->ldb, nullptr,
-                            h->stream));
+    a.labels_in = lin;
+    a.labels_out = lout;
+    CK(launch_km_operand(a, h->kp, h->stream));
     PartLayout ly;
     if ((rc = prod(h, nullptr, h->ntiles, nullptr, h->ntiles, h->P, &ly))) return rc;
     a.nsplit = ly.nsplit;
@@ -1472,16 +1477,12 @@ int symnmf_spkmeans(symnmf_t h, const int32_t *labels0, int32_t *labels, int32_t
     a.ncols = ly.ncols;
     CK(launch_km_centroids(a, h->kp, h->stream));
     // pass 2: P = S C, then the assignment
-    CK(launch_prepare_tiles(Hop, h->n, h->k, h->kp, h->Bt[h->cur], h->bt_fmt, h->ldb, nullptr,
-                            h->stream));
     if ((rc = prod(h, nullptr, h->ntiles, nullptr, h->ntiles, h->P, &ly))) return rc;
     a.nsplit = ly.nsplit;
     a.skG = ly.skG;
     a.ncols = ly.ncols;
-    a.labels_in = lin;
-    a.labels_out = lout;
     CK(launch_km_assign(a, h->kp, h->stream));
-    count_kernels(h, 6);
+    count_kernels(h, 5);
     CK(cudaMemcpyAsync(h->km_hout, h->km_out, 2 * sizeof(double), cudaMemcpyDeviceToHost,
                        h->stream));
     CK(cudaMemcpyAsync(h->host_err, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));

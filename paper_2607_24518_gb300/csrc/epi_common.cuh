@@ -64,10 +64,11 @@ __device__ __forceinline__ int64_t sk_cta(int64_t x, int64_t W, int64_t G) {
   return b;
 }
 
-// Partials of a product launch that ran without the fused epilogue: with
-// the stream-K layout (skG > 0) CTAs b0..b1 hold row position p's partials
-// in slots b + p; the SIMT layout has nsplit column shares per position.
-// part_sum adds the partials of row r, column c in that fixed order.
+// Partials of a product launch that ran without the fused epilogue (slots are
+// 128 x KP row-major blocks): with the stream-K layout (skG > 0) CTAs b0..b1
+// hold row position p's partials in slots b + p; the SIMT layout has nsplit
+// column shares per position, slot share * nlist + p.  They are added in that
+// order.
 __device__ __forceinline__ void part_range(int p, int skG, int ncols, int nlist, int64_t &b0,
                                            int64_t &b1) {
   b0 = b1 = 0;
@@ -77,18 +78,6 @@ __device__ __forceinline__ void part_range(int p, int skG, int ncols, int nlist,
     b1 = sk_cta((int64_t)p * ncols + ncols - 1, W, skG);
   }
 }
-template <int KP>
-__device__ __forceinline__ float part_sum(const float *P, int nsplit, int skG, int ncols, int nlist,
-                                          int p, int r, int c, int64_t b0, int64_t b1) {
-  float v = 0.f;
-  if (skG > 0) {
-    for (int64_t b = b0; b <= b1; ++b) v += P[((b + p) * kTileRows + r) * KP + c];
-  } else {
-    for (int s = 0; s < nsplit; ++s) v += P[(((int64_t)s * nlist + p) * kTileRows + r) * KP + c];
-  }
-  return v;
-}
-
 // num / (sqrt(v) + eps), the AdaGrad / RMSprop step (Sec. 2.2), in
 // straight-line code: PTX sqrt.approx.f32 (relative error at most 2^-23)
 // and div.full.f32 (at most 2 ulp over the full range).  With no

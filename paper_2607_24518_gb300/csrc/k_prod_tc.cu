@@ -222,7 +222,7 @@ __device__ __forceinline__ int unit_col(const TcArgs &a, int64_t L) {
 // and read by the epilogue warps of the same kernel only and are column-
 // major, so the 32 rows of a warp's load or store of one column are one
 // 128-byte line.  (Slots of a launch without the fused epilogue keep the
-// row-major layout of part_sum.)
+// row-major layout of part_range.)
 template <int KP>
 __device__ __forceinline__ int64_t fslot(int64_t s, int c, int r) {
   return (s * KP + c) * 128 + r;
