@@ -132,8 +132,9 @@ struct Cfg {
   static constexpr uint32_t BUDGET = 232448u - 1024u - BAR_BYTES - EPI_BYTES;
   // fewer stages than fit measured faster at kp = 64 (every storage type)
   // and with FP8 at kp = 32: about 120-130 KB in flight per SM; more only
-  // lengthens the round trips
-    static constexpr int STAGE_CAP = KP == 64 ? 4 : (F8 && KP == 32) ? 5 : 8;
+  // lengthens the round trips (FP32 at kp = 64 holds stages for three chains
+  // and takes the five that fit)
+  static constexpr int STAGE_CAP = KP == 64 ? (F32 ? 5 : 4) : (F8 && KP == 32) ? 5 : 8;
   static constexpr int STAGES = (BUDGET / STAGE) < (uint32_t)STAGE_CAP ? (int)(BUDGET / STAGE) : STAGE_CAP;
   static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE + BAR_BYTES + EPI_BYTES;
   // MMA issuing threads (warps 1 and 14).  One thread issues a tcgen05.mma
@@ -147,22 +148,22 @@ struct Cfg {
   // (SLO16: one bf16 S_lo buffer of 32 columns per ring stage, so a
   // stage's release also frees its S_lo buffer)
   static constexpr uint32_t ABUF = SLO16 ? 32u : F32 ? 32u * APS : 0u;
-  static constexpr int NABUF = SLO16 ? STAGES : F32 ? 2 : 1;
+  static constexpr int NABUF = SLO16 ? STAGES : F32 ? 4 : 1;
   static constexpr int NL = SLO16 ? N2 : 0;
   static constexpr uint32_t ACC0 = F32 ? NABUF * ABUF : 0u;
   static constexpr uint32_t ACCW = NA + NL;               // columns per accumulator buffer
-  static constexpr uint32_t PB0 = ACC0 + 2 * ACCW;        // double-buffered P rows
-  // kp = 64: the folders of BF16 and FP32 storage keep the running sum of a
-  // tile segment, or half of it, in tensor memory (PA) instead of 64
-  // registers per thread, which the 128-register budget of a 16-warp CTA
-  // cannot hold next to a fold's loads of two accumulators or the conversion
-  static constexpr bool PTMEM = (KP == 64);
+  // accumulator buffers, taken in turn by the chains
+  static constexpr int NACC = F32 && KP == 64 ? 4 : 2;
+  static constexpr uint32_t PB0 = ACC0 + NACC * ACCW;     // double-buffered P rows
+  // BF16 at kp = 64: the folders keep the running sum of a tile segment in
+  // tensor memory (PA) instead of 64 registers per thread, which the
+  // 128-register budget of a 16-warp CTA cannot hold next to a fold's loads of
+  // two accumulators.  FP8 and FP32, whose joined accumulator is all a fold
+  // reads, keep it in registers (FP8 step kernel at n = 20000, k = 64: 155 ->
+  // 144 us).
+  static constexpr bool PTMEM = (KP == 64 && DT == 1);
   static constexpr uint32_t PA0 = PB0 + 2 * KP;
-  // columns of the running sum kept in registers: with FP8, whose joined
-  // accumulator is all a fold reads, every one of them (step kernel at n =
-  // 20000, k = 64: 155 -> 144 us); FP32 half (1417 -> 1362 us at n = 30000),
-  // BF16 none (204 us either way)
-  static constexpr int NPR = !PTMEM || F8 ? KP : F32 ? KP / 2 : 0;
+  static constexpr int NPR = PTMEM ? 0 : KP;  // columns of the sum in registers
   static constexpr uint32_t TMEM_NEED = PA0 + (uint32_t)(KP - NPR);
   static constexpr uint32_t TMEM_COLS = TMEM_NEED <= 32 ? 32 : TMEM_NEED <= 64 ? 64 : TMEM_NEED <= 128 ? 128 : TMEM_NEED <= 256 ? 256 : 512;
   static_assert(STAGES >= 2, "shared memory ring too small");
@@ -1141,6 +1142,10 @@ __device__ void folder_role(const TcArgs &a, uint32_t tmem_base, uint8_t *smem, 
     const int ct = a.col_list ? a.col_list[ci] : ci;
     return __ldg(a.sS + (int64_t)rt * a.ld_sS + ct) * __ldg(a.deq + ct);
   };
+  // where the folders set the pace a whole-warp test first is quicker (n =
+  // 20000: FP32 k = 32 271 -> 266 us, FP8 k = 64 118 -> 113); FP8 below kp = 64
+  // and BF16 sleep in the wait (FP8 k = 32 83 against 85)
+  constexpr bool kReady = C::F32 || KP == 64 && C::F8;
   int64_t fcount = 0;  // units folded so far
   int fold_si = -1;     // segment of the last fold, and the end of its tile row
   int64_t tile_end = 0;
@@ -1163,7 +1168,8 @@ __device__ void folder_role(const TcArgs &a, uint32_t tmem_base, uint8_t *smem, 
       }
       ++fcount;
     }
-    if (!warp_wait(&tfull[acc], (tph >> acc) & 1u, abort_flag)) {
+    if (!(kReady ? warp_wait_ready(&tfull[acc], (tph >> acc) & 1u, abort_flag)
+                 : warp_wait(&tfull[acc], (tph >> acc) & 1u, abort_flag))) {
       fail(5);
       return;
     }
@@ -1275,60 +1281,36 @@ __device__ void folder_role(const TcArgs &a, uint32_t tmem_base, uint8_t *smem, 
   };
 
   if constexpr (C::F32) {
+    static_assert(C::SLO16, "kp = 64 has folder_role_wide");
     int stage = 0;
     uint32_t phase = 0;
-    uint32_t eph[4] = {0u, 0u, 0u, 0u};
     int64_t prev = -1, prev_hi = 0;  // chunk waiting to be folded
     int prev_si = 0;
-    int64_t run = 0;                  // chunks converted so far
     for (int si = 0; si < 2 && ok; ++si)
-    for (int64_t c = sg.lo[si] * C::SPU; c < sg.hi[si] * C::SPU && ok; ++c, ++run) {
-      const int ab = C::SLO16 ? stage : (int)(run % C::NABUF);
-      if (!warp_wait(&full[stage], phase, abort_flag) ||
-          (!C::SLO16 && !warp_wait(&aempty[ab], eph[ab] ^ 1, abort_flag))) {
+    for (int64_t c = sg.lo[si] * C::SPU; c < sg.hi[si] * C::SPU && ok; ++c) {
+      const int ab = stage;
+      if (!warp_wait_ready(&full[stage], phase, abort_flag)) {
         fail(15);
         break;
       }
       fence_after();
       const uint8_t *sa = smem + stage * C::STAGE;
-      if constexpr (C::SLO16) {
-        // S_lo = S - tf32_trunc(S) (exact), rounded to bf16, two per column
-#pragma unroll
-        for (int at = 0; at < C::APS; ++at) {
-          const uint8_t *rowp = sa + at * kAtomBytes + row * 128;
-          uint32_t pk[16];
-#pragma unroll
-          for (int ch = 0; ch < 8; ++ch) {  // 16-byte chunk of the 128-byte row
-            const float4 v = *reinterpret_cast<const float4 *>(rowp + ((ch ^ (row & 7)) << 4));
-            const __nv_bfloat162 l01 =
-                __floats2bfloat162_rn(v.x - tf32_trunc(v.x), v.y - tf32_trunc(v.y));
-            const __nv_bfloat162 l23 =
-                __floats2bfloat162_rn(v.z - tf32_trunc(v.z), v.w - tf32_trunc(v.w));
-            pk[2 * ch] = *reinterpret_cast<const uint32_t *>(&l01);
-            pk[2 * ch + 1] = *reinterpret_cast<const uint32_t *>(&l23);
-          }
-          tmem_st16(tmem_base + lane_off + (uint32_t)ab * C::ABUF + (uint32_t)at * 16u, pk);
-        }
-      } else
+      // S_lo = S - tf32_trunc(S) (exact), rounded to bf16, two per column
 #pragma unroll
       for (int at = 0; at < C::APS; ++at) {
         const uint8_t *rowp = sa + at * kAtomBytes + row * 128;
+        uint32_t pk[16];
 #pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {  // 16 columns at a time
-          uint32_t lo[16];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int ch = 4 * hh + j;  // 16-byte chunk of the 128-byte row
-            const float4 v = *reinterpret_cast<const float4 *>(rowp + ((ch ^ (row & 7)) << 4));
-            const float x[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-              lo[4 * j + u] = __float_as_uint(tf32_round(x[u] - tf32_trunc(x[u])));
-          }
-          tmem_st16(tmem_base + lane_off + (uint32_t)ab * C::ABUF + (uint32_t)at * 32u +
-                        (uint32_t)hh * 16u,
-                    lo);
+        for (int ch = 0; ch < 8; ++ch) {  // 16-byte chunk of the 128-byte row
+          const float4 v = *reinterpret_cast<const float4 *>(rowp + ((ch ^ (row & 7)) << 4));
+          const __nv_bfloat162 l01 =
+              __floats2bfloat162_rn(v.x - tf32_trunc(v.x), v.y - tf32_trunc(v.y));
+          const __nv_bfloat162 l23 =
+              __floats2bfloat162_rn(v.z - tf32_trunc(v.z), v.w - tf32_trunc(v.w));
+          pk[2 * ch] = *reinterpret_cast<const uint32_t *>(&l01);
+          pk[2 * ch + 1] = *reinterpret_cast<const uint32_t *>(&l23);
         }
+        tmem_st16(tmem_base + lane_off + (uint32_t)ab * C::ABUF + (uint32_t)at * 16u, pk);
       }
       tmem_wait_st();
       fence_before();
@@ -1337,7 +1319,6 @@ __device__ void folder_role(const TcArgs &a, uint32_t tmem_base, uint8_t *smem, 
         mbar_arrive(&empty[stage]);
         mbar_arrive(&afull[ab]);
       }
-      if constexpr (!C::SLO16) eph[ab] ^= 1;
       if (++stage == STAGES) {
         stage = 0;
         phase ^= 1;
@@ -1355,9 +1336,160 @@ __device__ void folder_role(const TcArgs &a, uint32_t tmem_base, uint8_t *smem, 
   }
 }
 
+// The folder warps of FP32 storage at kp = 64, where each stage is one chain
+// of 12 MMAs and the conversion and the fold of a stage cost these four warps
+// about what HBM takes to deliver it.  A stage is converted (S_lo to tensor
+// memory), then the stage three before it is folded, so the MMAs of three stages
+// are behind the one being converted (four accumulators and S_lo buffers) and
+// the folders wait for none of them; the loop has one copy of either, which
+// leaves room for the 64 sums in registers.  Step kernel without update at n =
+// 30000: 1362 -> 882 us (folding right after each conversion, half of the
+// sums in tensor memory, before); conversion, fold and their waits still take
+// about 1200 cycles per 16 KB stage, HBM 700.
+template <int KP>
+__device__ void folder_role_wide(const TcArgs &a, uint32_t tmem_base, uint8_t *smem, uint64_t *full,
+                                 uint64_t *empty, uint64_t *afull, uint64_t *aempty,
+                                 uint64_t *tfull, uint64_t *tempty, const Hand &hd,
+                                 volatile int *abort_flag, const Segs &sg, int b) {
+  using C = Cfg<0, KP>;
+  static_assert(C::APS == 1 && C::FOLD == 1 && C::NACC == 4 && C::NABUF == 4, "");
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int q = warp & 3, row = q * 32 + lane;
+  const uint32_t tlane = tmem_base + ((uint32_t)(q * 32) << 16);
+  float p[KP];
+#pragma unroll
+  for (int c = 0; c < KP; ++c) p[c] = 0.f;
+  int acc = 0, pb = 0, ab = 0, stage = 0;
+  uint32_t phase = 0, tph = 0u, pph = 0u, eph = 0u;  // bit i: parity of buffer i
+  auto fail = [&](int code) {
+    if (lane == 0) {
+      set_err(a.err, code);
+      *abort_flag = 1;
+    }
+    return false;
+  };
+  // a finished tile segment's P to the epilogue warps, or (without the fused
+  // epilogue) to row-major slot b + tp
+  auto finish = [&](int tp) -> bool {
+    if (a.fused) {
+      if (!warp_wait_idle(&hd.pempty[pb], ((pph >> pb) & 1u) ^ 1u, abort_flag)) return fail(7);
+      fence_after();
+#pragma unroll
+      for (int cc = 0; cc < KP; cc += 8) {
+        float v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = p[cc + j];
+        tmem_st8(tlane + C::PB0 + (uint32_t)(pb * KP + cc), v);
+      }
+      tmem_wait_st();
+      fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&hd.pfull[pb]);
+      pph ^= 1u << pb;
+      pb ^= 1;
+    } else {
+      float4 *dst = reinterpret_cast<float4 *>(a.out + ((int64_t)(b + tp) * 128 + row) * KP);
+#pragma unroll
+      for (int cc = 0; cc < KP; cc += 4)
+        dst[cc / 4] = make_float4(p[cc], p[cc + 1], p[cc + 2], p[cc + 3]);
+    }
+#pragma unroll
+    for (int c = 0; c < KP; ++c) p[c] = 0.f;
+    return true;
+  };
+  constexpr int CW = 16;  // accumulator columns per wait (32: 882 -> 926 us)
+  constexpr int LAG = 3;  // stages between conversion and fold
+  static_assert(LAG < C::NACC, "");
+  // position of the fold: units left in the segment and in its tile row
+  int si = sg.hi[0] > sg.lo[0] ? 0 : 1;
+  int seg_left = (int)(sg.hi[si] - sg.lo[si]);
+  int tp = (int)(sg.lo[si] / a.n_cols);
+  int left = (int)((int64_t)(tp + 1) * a.n_cols - sg.lo[si]);
+  int kc = 0;
+  const int total = (int)(sg.hi[0] - sg.lo[0] + sg.hi[1] - sg.lo[1]) * C::SPU;
+#pragma unroll 1
+  for (int it = 0; it < total + LAG; ++it) {
+    if (it < total) {
+      if (!warp_wait_ready(&full[stage], phase, abort_flag) ||
+          !warp_wait_ready(&aempty[ab], ((eph >> ab) & 1u) ^ 1u, abort_flag)) {
+        fail(15);
+        return;
+      }
+      fence_after();
+      const uint8_t *rowp = smem + stage * C::STAGE + row * 128;
+#pragma unroll
+      for (int hh = 0; hh < 2; ++hh) {  // 16 columns at a time
+        uint32_t lo[16];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int ch = 4 * hh + j;  // 16-byte chunk of the 128-byte row
+          const float4 v = *reinterpret_cast<const float4 *>(rowp + ((ch ^ (row & 7)) << 4));
+          const float w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            // the rounding increment of tf32_round; the MMA drops the low bits
+            lo[4 * j + i] = __float_as_uint(w[i] - tf32_trunc(w[i])) + 0x1000u;
+        }
+        tmem_st16(tlane + (uint32_t)ab * C::ABUF + (uint32_t)hh * 16u, lo);
+      }
+    }
+    if (it >= LAG && !warp_wait_ready(&tfull[acc], (tph >> acc) & 1u, abort_flag)) {
+      fail(5);
+      return;
+    }
+    if (it < total) {
+      tmem_wait_st();
+      fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(&empty[stage]);
+        mbar_arrive(&afull[ab]);
+      }
+      eph ^= 1u << ab;
+      ab = (ab + 1) & 3;
+      if (++stage == C::STAGES) {
+        stage = 0;
+        phase ^= 1u;
+      }
+    }
+    if (it < LAG) continue;
+    fence_after();
+    const uint32_t tb = tlane + C::ACC0 + (uint32_t)acc * C::ACCW;
+#pragma unroll
+    for (int cc = 0; cc < KP; cc += CW) {
+      uint32_t x[CW];
+#pragma unroll
+      for (int u = 0; u < CW; u += 8) tmem_ld8_nw(tb + (uint32_t)(cc + u), x, u);
+      tmem_wait_ld_all(x);
+#pragma unroll
+      for (int j = 0; j < CW; ++j) p[cc + j] += __uint_as_float(x[j]);
+    }
+    fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&tempty[acc]);
+    tph ^= 1u << acc;
+    acc = (acc + 1) & 3;
+    if (++kc < C::SPU) continue;
+    kc = 0;
+    --left;
+    --seg_left;
+    if ((left == 0 || seg_left == 0) && !finish(tp)) return;
+    if (left == 0) {
+      ++tp;
+      left = a.n_cols;
+    }
+    if (seg_left == 0 && si == 0) {
+      si = 1;
+      seg_left = (int)(sg.hi[1] - sg.lo[1]);
+      tp = (int)(sg.lo[1] / a.n_cols);
+      left = (int)((int64_t)(tp + 1) * a.n_cols - sg.lo[1]);
+    }
+  }
+}
+
 // MMA issuer `who` of NISSUE: issues the accumulator chains c with
 // c % NISSUE == who (chain c covers the CTA's stages [c FOLD, (c+1) FOLD)
-// and accumulates into buffer c % 2), commits each stage to its ring slot's
+// and accumulates into buffer c % NACC), commits each stage to its ring slot's
 // empty barrier and each finished chain to tfull.  The loop keeps its ring
 // position, phases and accumulator parities in registers and advances the
 // shared-memory descriptors by constant offsets: the issue rate of a single
@@ -1395,7 +1527,7 @@ __device__ __noinline__ void mma_role(const TcArgs &a, const Segs &sg, uint8_t *
       }
       continue;
     }
-    const int acc = (int)(c & 1);
+    const int acc = (int)(c % C::NACC);
     if (!mbar_wait(&tempty[acc], ((tph >> acc) & 1u) ^ 1u, abort_flag)) {
       set_err(a.err, 2);
       ok = false;
@@ -1513,8 +1645,8 @@ __global__ void __launch_bounds__(Cfg<DT, KP>::THREADS, 1)
   uint64_t *afull = empty + STAGES;
   uint64_t *aempty = afull + 8;
   uint64_t *tfull = aempty + 4;
-  uint64_t *tempty = tfull + 2;
-  uint64_t *pfull = tempty + 2;
+  uint64_t *tempty = tfull + 4;
+  uint64_t *pfull = tempty + 4;
   uint64_t *pempty = pfull + 2;
   uint64_t *drain = pempty + 2;  // one per MMA issuer
   uint32_t *holder = reinterpret_cast<uint32_t *>(drain + 2);
@@ -1533,9 +1665,11 @@ __global__ void __launch_bounds__(Cfg<DT, KP>::THREADS, 1)
     }
     for (int i = 0; i < 8; ++i) mbar_init(&afull[i], 4);
     for (int i = 0; i < 4; ++i) mbar_init(&aempty[i], 1);
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < 4; ++i) {
       mbar_init(&tfull[i], 1);
       mbar_init(&tempty[i], 4);
+    }
+    for (int i = 0; i < 2; ++i) {
       mbar_init(&pfull[i], 4);
       mbar_init(&pempty[i], 8);
     }
@@ -1626,8 +1760,12 @@ __global__ void __launch_bounds__(Cfg<DT, KP>::THREADS, 1)
     if (a.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   } else if (warp >= 10 && warp < 14) {
     const Hand hd{pfull, pempty, sflag};
-    folder_role<DT, KP>(a, tmem_base, smem, full, empty, afull, aempty, tfull, tempty, hd,
-                        abort_flag, sg, b, reinterpret_cast<float *>(scratch + 64));
+    if constexpr (C::F32 && C::JOIN)
+      folder_role_wide<KP>(a, tmem_base, smem, full, empty, afull, aempty, tfull, tempty, hd,
+                           abort_flag, sg, b);
+    else
+      folder_role<DT, KP>(a, tmem_base, smem, full, empty, afull, aempty, tfull, tempty, hd,
+                          abort_flag, sg, b, reinterpret_cast<float *>(scratch + 64));
   } else if (warp >= 2 && warp < 10) {
     const Hand hd{pfull, pempty, sflag};
     epilogue_role<DT, KP>(a, e, tmem_base, Hs, scratch, hd, abort_flag, sg);

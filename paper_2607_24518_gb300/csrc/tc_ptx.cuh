@@ -274,6 +274,12 @@ __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, volati
   if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, abort_flag) ? 1 : 0;
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
+// the same where the phase is usually complete: a test by the whole warp (no
+// branch, no shuffle), the bounded wait only if it fails
+__device__ __forceinline__ bool warp_wait_ready(uint64_t *bar, uint32_t parity,
+                                                volatile int *abort_flag) {
+  return __all_sync(0xffffffffu, mbar_test(bar, parity)) || warp_wait(bar, parity, abort_flag);
+}
 __device__ __forceinline__ bool warp_wait_idle(uint64_t *bar, uint32_t parity,
                                                volatile int *abort_flag) {
   int ok = 1;
