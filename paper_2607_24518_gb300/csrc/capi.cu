@@ -93,6 +93,7 @@ struct symnmf_ctx {
   size_t prof_used = 0;                // events used (2 per launch)
   double prof_bytes = 0.0;
   int64_t prof_kernels = 0;  // kernels launched by the solver loop while profiling
+  int batch_tiles = 0;       // row tiles of the batch being stepped (symnmf_batch_step)
   int ctas = 0;              // CTA cap of the tensor-core launches (0: all SMs)
   int restarts = 1;          // independent restarts concatenated along N
   // per-restart checks (restarts > 1): AND rule state and the last check
@@ -429,6 +430,7 @@ int prod(symnmf_t h, const int *row_list, int n_rows, const int *col_list, int n
   a.n_rows_list = n_rows;
   a.col_list = col_list;
   a.n_cols_list = n_cols;
+  a.batch_tiles = h->batch_tiles;
   a.out = out;
   const int64_t most = std::min<int64_t>(64, h->pq_cap_tiles / std::max(1, n_rows));
   const int ns = simt_shares(n_rows, n_cols, h->num_sms, (int)std::max<int64_t>(1, most));
@@ -1545,6 +1547,10 @@ int symnmf_batch_step(symnmf_t *hs, int32_t count, const symnmf_hparams *hps, in
       if (!first_err) first_err = rc;
     }
   }
+  int64_t tiles = 0;
+  for (int32_t i = 0; i < count; ++i) tiles += live[i] ? hs[i]->ntiles : 0;
+  for (int32_t i = 0; i < count; ++i)
+    if (live[i]) hs[i]->batch_tiles = (int)std::min<int64_t>(tiles, INT32_MAX);
   for (int32_t it = 0; it < iters; ++it) {
     // every live handle's iteration is launched before any check waits, so
     // one handle's check does not hold back the others' launches
@@ -1573,6 +1579,7 @@ int symnmf_batch_step(symnmf_t *hs, int32_t count, const symnmf_hparams *hps, in
   }
   for (int32_t i = 0; i < count; ++i) {
     if (!hs[i]) continue;
+    hs[i]->batch_tiles = 0;
     if (!hs[i]->bad) {
       symnmf_t h = hs[i];
       const int64_t upto = h->ctrl.converged ? h->ctrl.t + 1 : h->ctrl.t;

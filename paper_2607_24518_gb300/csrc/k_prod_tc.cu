@@ -134,7 +134,7 @@ struct Cfg {
   // and with FP8 at kp = 32: about 120-130 KB in flight per SM; more only
   // lengthens the round trips (FP32 at kp = 64 holds stages for three chains
   // and takes the five that fit)
-  static constexpr int STAGE_CAP = KP == 64 ? (F32 ? 5 : 4) : (F8 && KP == 32) ? 5 : 8;
+  static constexpr int STAGE_CAP = KP == 64 ? 5 : (F8 && KP == 32) ? 5 : 8;
   static constexpr int STAGES = (BUDGET / STAGE) < (uint32_t)STAGE_CAP ? (int)(BUDGET / STAGE) : STAGE_CAP;
   static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE + BAR_BYTES + EPI_BYTES;
   // MMA issuing threads (warps 1 and 14).  One thread issues a tcgen05.mma
@@ -1873,19 +1873,30 @@ cudaError_t launch_step_tc(const ProdArgs &a, const EpiArgs *epi, int *tile_cnt,
   TcArgs ta{};
   ta.W = (int64_t)a.n_rows_list * a.n_cols_list;
   ta.G = (int)std::max<int64_t>(1, std::min<int64_t>(ta.W, num_sms));
-  // A grid of m CTAs per row tile shares no CTA between two tiles (b W / G is
-  // then a tile boundary for every m-th b), so no CTA has to finish two tiles
-  // one after the other: an epilogue is 10 us, 20 at kp = 64.  Taken while the
-  // fuller shares cost less than that; a unit takes 0.5 (FP8) to 2 us (FP32; 4
-  // at kp = 64).  n = 4000: BF16 k = 8 / 32 / 64 24.5 / 46 / 87 -> 15.4 / 25 /
-  // 40 us, FP8 25 / 44 / 80 -> 16 / 26 / 44, FP32 k = 32 37 -> 31; n = 8000,
-  // k = 32: BF16 the same (36), FP8 41 -> 30; beyond the limits it loses (FP32
-  // n = 8000, 32 instead of 27 units: k = 16 56 -> 59, k = 64 131 -> 147).
+  // With fewer tiles than SMs the grid is m CTAs per row tile: b W / G is then
+  // a tile boundary for every m-th b, so no CTA holds parts of two tiles and
+  // finishes them one after the other (an epilogue is 10 us, 20 at kp = 64).
+  // m gives a CTA about `units` units; more CTAs per tile only add parts for
+  // the one that finishes it (iteration of BF16 n = 1000, k = 64: m = 8 47.6, m
+  // = 1 40.0 us; FP8 n = 2000, k = 64 52.5 -> 42.4; FP32 n = 2000, k = 64 53.4
+  // -> 50.5).  Where even the most CTAs leave longer shares than a full grid,
+  // the whole tiles are taken while the extra units cost less than an epilogue
+  // (n = 4000: BF16 k = 8 / 32 / 64 24.5 / 46 / 87 -> 15.4 / 25 / 40 us, FP8
+  // 25 / 44 / 80 -> 16 / 26 / 44; beyond the limits it loses: FP32 n = 8000,
+  // 32 instead of 27 units, k = 16 56 -> 59, k = 64 131 -> 147).
+  // Handles stepped together share the SMs: m is such that all their tiles make
+  // two grids, so that small ones run side by side (8 handles n <= 8000 k = 16
+  // BF16 1826 -> 1630 us for ten iterations, 8 of n <= 4000 k = 32 FP32 1897 ->
+  // 1477; one grid in all: 2 of n <= 6000 720 -> 953).
   if (epi && a.n_rows_list < num_sms) {
-    const int m = std::min(num_sms / a.n_rows_list, a.n_cols_list);
-    const int whole = (a.n_cols_list + m - 1) / m, share = (int)((ta.W + ta.G - 1) / ta.G);
-    const int most = a.dtype == 0 ? (a.kp == 64 ? 0 : 3) : a.kp == 64 ? 3 : 8;
-    if (whole - share <= most) ta.G = m * a.n_rows_list;
+    const int R = a.n_rows_list, cols = a.n_cols_list;
+    const int most = std::min(num_sms / R, cols);
+    const int units = a.dtype == 0 ? 4 : a.dtype == 1 ? 12 : a.kp == 64 ? 20 : 14;
+    int m = std::min(most, (cols + units - 1) / units);
+    if (a.batch_tiles > R) m = std::max(1, std::min(m, 2 * num_sms / a.batch_tiles));
+    const int whole = (cols + m - 1) / m, share = (int)((ta.W + ta.G - 1) / ta.G);
+    const int extra = a.dtype == 0 ? (a.kp == 64 ? 0 : 3) : a.dtype == 1 && a.kp == 64 ? 3 : 8;
+    if (m < most || whole - share <= extra) ta.G = m * R;
   }
   ta.n_cols = a.n_cols_list;
   ta.row_list = a.row_list;
@@ -1893,10 +1904,11 @@ cudaError_t launch_step_tc(const ProdArgs &a, const EpiArgs *epi, int *tile_cnt,
   ta.out = a.out;
   ta.err = err;
   ta.fused = (epi != nullptr) ? 1 : 0;
-  // early only when the grid leaves an SM to every block of the reduction:
-  // otherwise its blocks pile up on the first SMs that CTAs leave, which then
-  // start the next step late (n = 20000, k = 32: +11 us an iteration)
-  ta.early = ta.fused && ta.G + 1 + a.kp * a.kp / 16 <= num_sms;
+  // early only when the grid leaves an SM to every block of the reduction and
+  // no other handle's step wants them: otherwise its blocks pile up on the
+  // first SMs that CTAs leave, which then start the next step late (n = 20000,
+  // k = 32: +11 us an iteration; 8 handles n <= 4000 FP32 1477 -> 1650)
+  ta.early = ta.fused && a.batch_tiles <= a.n_rows_list && ta.G + 1 + a.kp * a.kp / 16 <= num_sms;
   ta.tile_cnt = tile_cnt;
   // every row position shared stream-K style (owning whole tiles makes the
   // leftover tiles' last arrivers add ~G / R partials each while HBM is

@@ -80,6 +80,7 @@ struct ProdArgs {
   const int *col_list;   // column tile indices (nullptr: all tiles in order)
   int n_cols_list;
   int nsplit;
+  int batch_tiles;       // row tiles of all handles stepped together (0: one handle)
   float *out;
 };
 
