@@ -121,7 +121,7 @@ struct Cfg {
   // FP32 registers
   static constexpr int FOLD = F32 ? 1 : SPU;
   // accumulator columns per part read before one wait when folding
-  static constexpr int FOLD_CW = F32 ? 8 : (KP == 64 ? 16 : 32);
+    static constexpr int FOLD_CW = F32 ? 8 : (KP == 64 ? 16 : 32);
   // the epilogue's H tile (kp = 64: and a second tile-shaped buffer for
   // H_t Gram_t and then g, which 32 columns per thread cannot keep in
   // registers); the Gram of H_t is read from global memory (L1)
@@ -152,8 +152,11 @@ struct Cfg {
   static constexpr int NL = SLO16 ? N2 : 0;
   static constexpr uint32_t ACC0 = F32 ? NABUF * ABUF : 0u;
   static constexpr uint32_t ACCW = NA + NL;               // columns per accumulator buffer
-  // accumulator buffers, taken in turn by the chains
-  static constexpr int NACC = F32 && KP == 64 ? 4 : 2;
+  // accumulator buffers, taken in turn by the chains: four where tensor
+  // memory holds them, so that a late fold holds the MMAs up less (against
+  // two, n = 20000: FP8 k = 16 / 32 / 64 74.8 / 83.2 / 112.3 -> 70.7 / 80.7 /
+  // 109.6 us, BF16 k = 16 128 -> 126, k = 32 134.3 -> 133.3)
+  static constexpr int NACC = F32 ? (KP == 64 ? 4 : 2) : F8 || KP <= 32 ? 4 : 2;
   static constexpr uint32_t PB0 = ACC0 + NACC * ACCW;     // double-buffered P rows
   // BF16 at kp = 64: the folders keep the running sum of a tile segment in
   // tensor memory (PA) instead of 64 registers per thread, which the
@@ -1266,7 +1269,7 @@ __device__ void folder_role(const TcArgs &a, uint32_t tmem_base, uint8_t *smem, 
     __syncwarp();
     if (lane == 0) mbar_arrive(&tempty[acc]);
     tph ^= 1u << acc;
-    acc ^= 1;
+    acc = acc + 1 == C::NACC ? 0 : acc + 1;
     const int64_t cend = (f + 1) * C::FOLD;
     if (cend % C::SPU == 0) {
       const int64_t u = cend / C::SPU - 1;  // unit just completed
