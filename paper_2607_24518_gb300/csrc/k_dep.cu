@@ -33,10 +33,10 @@
 // FP16 pieces hold as many bits as tf32 ones (11) in half the bytes and at
 // twice the tensor rate, and a dot product takes half as many chained
 // accumulations; the column scales remove FP16's narrow range.  n = 20000,
-// T = 500: FP32 / BF16 / FP8 output 687 / 538 / 463 us (tf32 pieces, four
+// T = 500: FP32 / BF16 / FP8 output 548 / 462 / 442 us (tf32 pieces, four
 // epilogue warps with per-entry tests and stores: 1348 / 1349 / 2102 us),
 // error of S 1.8e-6 instead of 4.5e-6.  The FP8 figure is the operand
-// stream's (4.8 GB from L2, 10 TB/s); the wider outputs add their stores.
+// stream's (4.8 GB from L2, 11 TB/s); the wider outputs add their stores.
 // Every mbarrier wait is bounded (2 s); on expiry the CTA records an error
 // code, drains its own copies, frees its tensor memory and returns.
 #include <cuda.h>
@@ -186,6 +186,7 @@ struct DepArgs {
   int64_t ld_scales;
   double *sq;       // per CTA
   int *err;
+  bool w8;          // every row of S starts on a 32-byte boundary
   int exact_sq;     // F32 / BF16: run sums of squares as float-float pairs
 };
 
@@ -238,6 +239,23 @@ __device__ __forceinline__ bool dep_all(int h, bool ok) {
       : "r"(1 + h), "r"((uint32_t)ok)
       : "memory");
   return r != 0;
+}
+// 32 bytes of one row, on a 32-byte boundary when w8, else on a 16-byte one.
+// The rows of a warp lie in 32 lines; a 16-byte store is a partial sector to
+// L2, which bounded the wider outputs (n = 20000, T = 500, GEMM: FP32 684 ->
+// 548 us, BF16 535 -> 462, FP8 462 -> 442; streaming and write-through hints
+// changed nothing).
+__device__ __forceinline__ void dep_store32(void *dst, bool w8, uint32_t a, uint32_t b, uint32_t c,
+                                            uint32_t d, uint32_t e, uint32_t f, uint32_t g,
+                                            uint32_t h) {
+  if (w8) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(a),
+                 "r"(b), "r"(c), "r"(d), "r"(e), "r"(f), "r"(g), "r"(h)
+                 : "memory");
+  } else {
+    reinterpret_cast<uint4 *>(dst)[0] = make_uint4(a, b, c, d);
+    reinterpret_cast<uint4 *>(dst)[1] = make_uint4(e, f, g, h);
+  }
 }
 // barrier among the 128 epilogue threads of column half h
 __device__ __forceinline__ void dep_bar(int h) {
@@ -462,9 +480,7 @@ __global__ void __launch_bounds__(kDepThreads, 1)
           for (int u = 0; u < 32; ++u) part = fmaf(wgt(c0 + u) * v[u], v[u], part);
           sq += (double)part;
           if (inner) {
-            uint4 *dst = reinterpret_cast<uint4 *>(Srow + j0 + c0);
-            dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
-            dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+            dep_store32(Srow + j0 + c0, a.w8, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
             // mirror: 4 x 4 byte transposes among the lanes 4 p + z, after
             // which lane 4 p + z holds column c0 + 4 u + z of rows 4 p ..
             // 4 p + 3, one word of S's row j
@@ -522,9 +538,11 @@ __global__ void __launch_bounds__(kDepThreads, 1)
             if (inner) {
               float *Scol = S32 + (j0 + c0) * a.lds + i;
 #pragma unroll
-              for (int u = 0; u < 8; ++u)
-                reinterpret_cast<float4 *>(Srow)[u] =
-                    make_float4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
+              for (int u = 0; u < 32; u += 8)
+                dep_store32(Srow + u, a.w8, __float_as_uint(v[u]), __float_as_uint(v[u + 1]),
+                            __float_as_uint(v[u + 2]), __float_as_uint(v[u + 3]),
+                            __float_as_uint(v[u + 4]), __float_as_uint(v[u + 5]),
+                            __float_as_uint(v[u + 6]), __float_as_uint(v[u + 7]));
 #pragma unroll
               for (int u = 0; u < 32; ++u) Scol[u * a.lds] = v[u];
             } else if (vrow) {
@@ -543,9 +561,9 @@ __global__ void __launch_bounds__(kDepThreads, 1)
               for (int u = 0; u < 16; ++u)
                 w[u] = (__float_as_uint(v[2 * u]) >> 16) | (__float_as_uint(v[2 * u + 1]) & 0xFFFF0000u);
 #pragma unroll
-              for (int u = 0; u < 4; ++u)
-                reinterpret_cast<uint4 *>(Srow)[u] =
-                    make_uint4(w[4 * u], w[4 * u + 1], w[4 * u + 2], w[4 * u + 3]);
+              for (int u = 0; u < 16; u += 8)
+                dep_store32(Srow + 2 * u, a.w8, w[u], w[u + 1], w[u + 2], w[u + 3], w[u + 4],
+                            w[u + 5], w[u + 6], w[u + 7]);
               // mirror: 2 x 2 transposes among lane pairs, then lane z of a
               // pair holds column c0 + 2 u + z of the pair's two rows
               const int z = lane & 1;
@@ -677,6 +695,7 @@ cudaError_t launch_dependence(const float *Y, int64_t T, int64_t n, int64_t ldy,
     a.sq = sq;
     a.err = err;
     a.exact_sq = exact_norm ? 1 : 0;
+    a.w8 = reinterpret_cast<uintptr_t>(S) % 32 == 0 && (lds * (out == 0 ? 4 : out == 1 ? 2 : 1)) % 32 == 0;
     dep_gemm_kernel<<<(unsigned)G, kDepThreads, kDepSmem, s>>>(mP, a);
     if (normS2) dep_sum_kernel<<<1, 256, 0, s>>>(sq, G, normS2);
     e = cudaGetLastError();

@@ -80,3 +80,24 @@ def test_tile_list_and_mirrors(L, T, n, out):
         assert float((got - ref).abs().max()) <= bound
     assert torch.equal(got, got.T)
     assert bool((S[:, n:].float() == 77).all())
+
+
+@pytest.mark.parametrize("out,es", [("f32", 4), ("bf16", 2), ("fp8", 1)])
+def test_rows_on_16_but_not_on_32_bytes(L, out, es):
+    """Rows on 16-byte boundaries only take 16-byte stores: the same entries
+    as with rows on 32-byte boundaries."""
+    T, n = 64, 300
+    Y = torch.tensor(np.random.default_rng(3).standard_normal((T, n)), dtype=torch.float32, device=DEV)
+    dt = {"f32": torch.float32, "bf16": torch.bfloat16, "fp8": torch.uint8}[out]
+    got = []
+    for pitch, off in ((320 * 4, 0), (320 * 4 + 16, 0), (320 * 4, 16)):
+        lds = pitch // es
+        flat = torch.zeros(n * lds + 64, dtype=dt, device=DEV)
+        S = flat[off // es:off // es + n * lds].view(n, lds)
+        sc = torch.zeros(3, 3, device=DEV)
+        L.symnmf_build_dependence(Y, T, n, n, 1, {"f32": L.F32, "bf16": L.BF16, "fp8": L.FP8E4M3}[out],
+                                  S, lds, sc, 3)
+        got.append((S[:, :n].float(), sc))
+        assert not bool((S[:, n:].float() != 0).any())
+    for S, sc in got[1:]:
+        assert torch.equal(S, got[0][0]) and torch.equal(sc, got[0][1])
