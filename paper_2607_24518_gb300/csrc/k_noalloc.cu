@@ -80,7 +80,7 @@ __device__ void gram_tile(const ObjArgs &a, int tile, float *sm) {
 }
 
 // blockIdx.y < split: a column share; == split: the tile's Gram partial.
-// n = 10000, KP = 32 FP32: 500 -> 244 us (13 TFMA/s of 37); the tile Grams
+// n = 10000, KP = 32 FP32: 500 -> 188 us (17 TFMA/s of 37); the tile Grams
 // beside the shares and their sum over the chip replace a pass of their own
 // and one CTA's 49 us.
 template <int DT, int KP>

@@ -10,7 +10,7 @@
 namespace symnmf {
 namespace {
 
-// 128 registers for two CTAs per SM.  n = 3001, KP = 16 FP32 33 -> 16 us; n =
+// 128 registers for two CTAs per SM.  n = 3001, KP = 16 FP32 33 -> 15 us; n =
 // 5001, KP = 32 BF16 94 -> 57 us (one 16-value block per thread fed by scalar
 // reads, no chunk in flight during the FMAs, before).
 template <int DT, int KP>

@@ -9,7 +9,7 @@
 // threads split each 32-column chunk among NG such groups, whose sums are
 // added in group order at the end.  FP32 chunks arrive by cp.async in a ring
 // of four (one chunk ahead in registers waited on HBM's latency: n = 10000,
-// KP = 32 301 -> 244 us); BF16 and FP8 entries, of any byte alignment, are
+// KP = 32 301 -> 244 us; rows on 16-byte boundaries in 16-byte pieces: 188 us); BF16 and FP8 entries, of any byte alignment, are
 // loaded one chunk ahead into registers and widened there (staged as aligned
 // words and widened in shared memory: n = 5001, KP = 32 60 -> 77 us).
 #pragma once
@@ -37,7 +37,8 @@ struct Simt {
   static constexpr int LD = BK + 4;              // FP32 rows: 16-byte aligned, no bank conflicts
   static constexpr int S_WORDS = 128 * LD;       // FP32 tile
   static constexpr int BUFS = DT == 0 ? RING : 2;
-  static constexpr int STAGE = S_WORDS + BK * KP;  // S chunk, H chunk
+  static constexpr int H_WORDS = BK * KP;
+  static constexpr int STAGE = S_WORDS + H_WORDS;  // S chunk, H chunk
   static constexpr int WORDS = BUFS * STAGE;
   static constexpr size_t SMEM = sizeof(float) * WORDS;
   static_assert(KG % 2 == 0 && 128 * KP <= WORDS && STAGE % 4 == 0, "");
@@ -46,6 +47,14 @@ struct Simt {
 // 4 bytes to shared memory, the first `bytes` (0..4) from src and zeros after
 __device__ __forceinline__ void cp_async4(float *dst, const void *src, int bytes) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                   static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+               "l"(src), "r"(bytes)
+               : "memory");
+}
+
+// the same for 16 bytes (0..16 from src), both addresses on 16-byte boundaries
+__device__ __forceinline__ void cp_async16(float *dst, const void *src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
                    static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
                "l"(src), "r"(bytes)
                : "memory");
@@ -77,23 +86,46 @@ __device__ __forceinline__ void simt_tile(float *sm, const void *S, int64_t lds,
     const int ci = cb + (q >> 2);
     return (int64_t)(col_list ? col_list[ci] : ci) * kTileRows + (q & 3) * C::BK;
   };
-  // FP32: chunk q into its stage of the ring
+  // FP32: chunk q into its stage of the ring, 16 bytes at a time where every
+  // row of S (H) starts on such a boundary
+  const bool svec = reinterpret_cast<uintptr_t>(S) % 16 == 0 && lds % 4 == 0;
+  const bool hvec = reinterpret_cast<uintptr_t>(H) % 16 == 0 && ldh == KP && k == KP;
   auto issue = [&](int q) {
     if (q < nq) {
       const int64_t c0 = col0(q);
       const int cols = (int)(n - c0 < C::BK ? n - c0 : C::BK);  // may be <= 0
       float *st = sm + (q % C::RING) * C::STAGE, *hs = st + C::S_WORDS;
-      const float *p = reinterpret_cast<const float *>(S) + (r0 + warp) * lds + c0 + lane;
-#pragma unroll 4
-      for (int r = warp; r < 128; r += 8, p += 8 * lds) {
-        const bool in = r < rows && lane < cols;
-        cp_async4(st + r * C::LD + lane, in ? (const void *)p : S, in ? 4 : 0);
-      }
+      const float *Sf = reinterpret_cast<const float *>(S);
+      if (svec) {  // 4 columns per thread, rows tid / 8, + 32, ...
+        const int c4 = 4 * (tid & 7);
+        const int bytes = cols - c4 >= 4 ? 16 : cols > c4 ? 4 * (cols - c4) : 0;
+        const float *p = Sf + (r0 + (tid >> 3)) * lds + c0 + c4;
 #pragma unroll
-      for (int i = 0; i < HV; ++i) {
-        const int e = tid + 256 * i, r = e / KP, c = e % KP;
-        const bool in = r < cols && c < k;
-        cp_async4(hs + e, in ? H + (c0 + r) * ldh + c : H, in ? 4 : 0);
+        for (int i = 0; i < 4; ++i, p += 32 * lds) {
+          const int r = (tid >> 3) + 32 * i;
+          const int nb = r < rows ? bytes : 0;
+          cp_async16(st + r * C::LD + c4, nb ? (const void *)p : S, nb);
+        }
+      } else {
+        const float *p = Sf + (r0 + warp) * lds + c0 + lane;
+#pragma unroll 4
+        for (int r = warp; r < 128; r += 8, p += 8 * lds) {
+          const bool in = r < rows && lane < cols;
+          cp_async4(st + r * C::LD + lane, in ? (const void *)p : S, in ? 4 : 0);
+        }
+      }
+      if (hvec) {
+        for (int e = 4 * tid; e < C::H_WORDS; e += 1024) {
+          const int r = e / KP, c = e % KP;
+          cp_async16(hs + e, r < cols ? H + (c0 + r) * KP + c : H, r < cols ? 16 : 0);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < HV; ++i) {
+          const int e = tid + 256 * i, r = e / KP, c = e % KP;
+          const bool in = r < cols && c < k;
+          cp_async4(hs + e, in ? H + (c0 + r) * ldh + c : H, in ? 4 : 0);
+        }
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
