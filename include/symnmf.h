@@ -249,9 +249,10 @@ int symnmf_batch_step(symnmf_t *hs, int32_t count, const symnmf_hparams *hps, in
                       symnmf_stats *outs);
 /* Cap the CTAs of the handle's tensor-core launches (0 = one per SM, the
  * default; a matrix of fewer than 128 rows per SM may take fewer, and fewer
- * still while it is stepped with others).  Several handles with small caps on different streams run
- * their iterations side by side (batching: symnmf_batch_step).  This
- * library's scheduling knob; the paper runs one solve at a time. */
+ * still while it is stepped with others).  Several handles with small caps
+ * on different streams run their iterations side by side (batching:
+ * symnmf_batch_step).  This library's scheduling knob; the paper runs one
+ * solve at a time. */
 int symnmf_set_ctas(symnmf_t h, int32_t ctas);
 /* The most CTAs the handle's launches use (host). */
 int symnmf_get_ctas(symnmf_t h, int32_t *ctas);

@@ -6,18 +6,21 @@
 //   warp 0      TMA producer: streams 128-row tiles of S (128-byte swizzled
 //               atoms) and the matching slice of the hi/lo MMA copy of H^T
 //               into a ring of shared-memory stages
-//   warp 1      MMA issuer: one thread issues tcgen05.mma into a double-
-//               buffered 128 x 2kp TMEM accumulator (columns [0,kp) multiply
-//               H_hi, [kp,2kp) multiply H_lo) and frees stages with
-//               tcgen05.commit
+//   warps 1, 14 MMA issuers: one thread of each issues tcgen05.mma for
+//               alternate chains into two or four TMEM accumulators in turn
+//               (128 x 2kp: columns [0,kp) multiply H_hi, [kp,2kp) multiply
+//               H_lo; 128 x kp where both parts share the columns) and frees
+//               stages with tcgen05.commit
 //   warps 2-9   epilogue, two threads per tile row (half the columns each):
-//               (tcgen05.ld), P = acc_hi + acc_lo, and for a finished tile
-//               runs the whole per-row update: g = 4 (H Gram_t - P), the
+//               reads P from the folders' hand-over block (tcgen05.ld) and for
+//               a finished tile runs the whole per-row update:
+//               g = 4 (H Gram_t - P), the
 //               AdaGrad / RMSprop / ADMM step with the max(0, .) projection
 //               into the other H buffer, the MMA copy of the new rows, and
 //               the tile partials tr = sum H * P, ||grad_proj||^2, sum(G),
 //               NaN count and the Gram partial H'^T H'
-//   warps 10-13 folders: fold each accumulator chain into FP32 registers and
+//   warps 10-13 folders: fold each accumulator chain into FP32 (registers;
+//               BF16 at kp = 64: tensor memory) and
 //               hand a finished tile segment's P over; with FP32 storage
 //               they also convert the staged S rows, see below; with FP8
 //               storage they apply the per-unit scale of S when folding
@@ -41,7 +44,8 @@
 //         applied per unit when the folders fold
 // Work: the row-major list of (row tile, 128-column tile) units is split
 // into equal contiguous ranges, one per CTA (stream-K), so every SM streams
-// the same number of S bytes.  A tile whose units span several CTAs is
+// the same number of S bytes (grids of fewer tiles than SMs take a whole
+// number of CTAs per tile).  A tile whose units span several CTAs is
 // finished by the last of them to arrive (per-tile counter): the others
 // leave their FP32 partial in slot (cta + tile); the finisher adds the
 // slots in CTA order, so results do not depend on timing.  Finished tiles
@@ -121,7 +125,7 @@ struct Cfg {
   // FP32 registers
   static constexpr int FOLD = F32 ? 1 : SPU;
   // accumulator columns per part read before one wait when folding
-    static constexpr int FOLD_CW = F32 ? 8 : (KP == 64 ? 16 : 32);
+  static constexpr int FOLD_CW = F32 ? 8 : (KP == 64 ? 16 : 32);
   // the epilogue's H tile (kp = 64: and a second tile-shaped buffer for
   // H_t Gram_t and then g, which 32 columns per thread cannot keep in
   // registers); the Gram of H_t is read from global memory (L1)

@@ -9,9 +9,10 @@
 // threads split each 32-column chunk among NG such groups, whose sums are
 // added in group order at the end.  FP32 chunks arrive by cp.async in a ring
 // of four (one chunk ahead in registers waited on HBM's latency: n = 10000,
-// KP = 32 301 -> 244 us; rows on 16-byte boundaries in 16-byte pieces: 188 us); BF16 and FP8 entries, of any byte alignment, are
-// loaded one chunk ahead into registers and widened there (staged as aligned
-// words and widened in shared memory: n = 5001, KP = 32 60 -> 77 us).
+// KP = 32 301 -> 244 us; rows on 16-byte boundaries in 16-byte pieces: 188 us);
+// BF16 and FP8 entries, of any byte alignment, are loaded one chunk ahead into
+// registers and widened there (staged as aligned words and widened in shared
+// memory: n = 5001, KP = 32 60 -> 77 us).
 #pragma once
 #include "epi_common.cuh"
 
