@@ -429,7 +429,9 @@ __global__ void __launch_bounds__(256) reduce_iter_kernel(ReduceArgs a) {
 }
 
 // Gram of the tiles of a list, 16 threads to an entry as in reduce_iter_kernel
-// (one thread per entry: 391 tiles at kp = 64 47 us, now 17)
+// (one thread per entry: 391 tiles at kp = 64 47 us, now 17).  It runs in the
+// tail of the products before it, of which it needs nothing, and waits for
+// them before it ends, as the epilogue that follows needs both.
 template <int KP>
 __global__ void __launch_bounds__(256) gram_subset_kernel(const float *gram_part, const int *l1,
                                                           int n1, const int *l2, int n2,
@@ -456,6 +458,7 @@ __global__ void __launch_bounds__(256) gram_subset_kernel(const float *gram_part
 #pragma unroll
   for (int i = 0; i < 16; ++i) s += red[i * 16 + tid];
   if (kb > 0 && e / KP / kb != e % KP / kb) s = 0.0;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   (blockIdx.y == 0 ? o1 : o2)[e] = (float)s;
 }
 
@@ -696,9 +699,18 @@ cudaError_t launch_reduce_iter(const ReduceArgs &a, int kp, cudaStream_t s) {
 
 cudaError_t launch_gram_subset(const float *gram_part, int kp, const int *l1, int n1,
                                const int *l2, int n2, float *o1, float *o2, int kb, cudaStream_t s) {
-  dim3 grid(kp * kp / 16, 2);
-  KP_SWITCH(kp, gram_subset_kernel<KPV><<<grid, 256, 0, s>>>(gram_part, l1, n1, l2, n2, o1, o2, kb));
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kp * kp / 16, 2);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  KP_SWITCH(kp, return cudaLaunchKernelEx(&cfg, gram_subset_kernel<KPV>, gram_part, l1, n1, l2, n2,
+                                          o1, o2, kb));
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_norm_s2(const void *S, int64_t n, int64_t lds, int dtype, const float *scales,

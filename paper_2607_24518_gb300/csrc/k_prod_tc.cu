@@ -85,6 +85,7 @@ struct TcArgs {
   int *err;
   int fused;             // run the per-tile epilogue in the kernel
   int early;             // let the reduction kernel launch before this grid ends
+  int chain;             // Chain bits (not fused)
   int *tile_cnt;         // per-tile arrival counters (fused)
   const float *sS;       // FP8: tile scales of S (row pitch ld_sS)
   int64_t ld_sS;
@@ -796,7 +797,11 @@ __device__ void epilogue_role(const TcArgs &a, const EpiArgs &e, uint32_t tmem_b
   const int et = (warp - 2) * 32 + lane;  // 0..255
   const int half = (warp - 2) >> 2;       // column half owned
   float *Gx = Hs + 128 * (KP + 1);        // kp = 64 only (Own<KP>::GX)
-  if (!a.fused) return;
+  if (!a.fused) {
+    // what waits for this grid has waited for the one it overlaps, too
+    if (a.chain & CHAIN_NEXT) asm volatile("griddepcontrol.wait;" ::: "memory");
+    return;
+  }
   // the Gram of H_t and the tile slots belong to the preceding reduction
   // kernel, which may still run (programmatic dependent launch).  The Gram
   // is read from global memory: its next writer is the reduction kernel
@@ -1694,6 +1699,9 @@ __global__ void __launch_bounds__(Cfg<DT, KP>::THREADS, 1)
   const int b = blockIdx.x;
   const Segs sg = cta_segments(a, b);
   int issued = 0;
+  // a CTA takes all registers of its SM, so the next launch's CTAs start one
+  // by one as this one's leave, or on SMs that this grid does not use
+  if (a.chain & CHAIN_HEAD) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
     if (lane == 0) {
@@ -1835,7 +1843,7 @@ cudaError_t launch_cfg(const ProdArgs &p, const EpiArgs &e, cudaStream_t s, cons
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = ta.fused ? 1 : 0;
+  cfg.numAttrs = ta.fused || (ta.chain & CHAIN_NEXT) ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, step_tc_kernel<DT, KP>, mS, mB, mB2, ta, e);
 }
 
@@ -1916,6 +1924,7 @@ cudaError_t launch_step_tc(const ProdArgs &a, const EpiArgs *epi, int *tile_cnt,
   // first SMs that CTAs leave, which then start the next step late (n = 20000,
   // k = 32: +11 us an iteration; 8 handles n <= 4000 FP32 1477 -> 1650)
   ta.early = ta.fused && a.batch_tiles <= a.n_rows_list && ta.G + 1 + a.kp * a.kp / 16 <= num_sms;
+  ta.chain = ta.fused ? 0 : a.chain;
   ta.tile_cnt = tile_cnt;
   // every row position shared stream-K style (owning whole tiles makes the
   // leftover tiles' last arrivers add ~G / R partials each while HBM is

@@ -81,7 +81,13 @@ struct ProdArgs {
   int n_cols_list;
   int nsplit;
   int batch_tiles;       // row tiles of all handles stepped together (0: one handle)
+  int chain;             // Chain bits: products of one iteration that need nothing of each other
   float *out;
+};
+
+enum Chain {
+  CHAIN_HEAD = 1,  // the next launch may start as this one's CTAs leave their SMs
+  CHAIN_NEXT = 2,  // launched so: waits for the launch before it only before it ends
 };
 
 // Partial-sum layout of a product launch: split layout (SIMT: nsplit
