@@ -1489,13 +1489,20 @@ int symnmf_spkmeans(symnmf_t h, const int32_t *labels0, int32_t *labels, int32_t
     a.labels_out = lout;
     CK(launch_km_operand(a, h->kp, h->stream));
     PartLayout ly;
-    if ((rc = prod(h, nullptr, h->ntiles, nullptr, h->ntiles, h->P, &ly))) return rc;
+    if ((rc = prod(h, nullptr, h->ntiles, nullptr, h->ntiles, h->P, &ly, nullptr, CHAIN_AFTER)))
+      return rc;
     a.nsplit = ly.nsplit;
     a.skG = ly.skG;
     a.ncols = ly.ncols;
     CK(launch_km_centroids(a, h->kp, h->stream));
     // pass 2: P = S C, then the assignment
-    if ((rc = prod(h, nullptr, h->ntiles, nullptr, h->ntiles, h->P, &ly))) return rc;
+    if ((rc = prod(h, nullptr, h->ntiles, nullptr, h->ntiles, h->P, &ly, nullptr,
+                   CHAIN_AFTER | CHAIN_HEAD)))
+      return rc;
+    // the norms belong to the assignment: beside the product instead of
+    // before it.  With the launches as programmatic dependents five iterations
+    // at n = 20000, K = 32 BF16 take 1429 instead of 1510 us
+    CK(launch_km_norms(a, h->kp, h->stream));
     a.nsplit = ly.nsplit;
     a.skG = ly.skG;
     a.ncols = ly.ncols;

@@ -11,6 +11,23 @@
 
 namespace symnmf {
 
+// Launch as a programmatic dependent of the kernel before it in the stream:
+// the kernel executes griddepcontrol.wait before it touches what that one
+// writes, and always before it ends.
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*f)(P...), dim3 grid, int threads, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, f, args...);
+}
+
 __device__ __forceinline__ uint16_t bf16_bits(float x) {
   __nv_bfloat16 b = __float2bfloat16_rn(x);
   return *reinterpret_cast<uint16_t *>(&b);

@@ -662,16 +662,7 @@ cudaError_t launch_epilogue(const EpiArgs &a, cudaStream_t s) {
 
 cudaError_t launch_admm_minv(const double *gram64, int k, int kp, double rho, float *minv,
                              cudaStream_t s) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(1);
-  cfg.blockDim = dim3(256);
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  KP_SWITCH(kp, return cudaLaunchKernelEx(&cfg, admm_minv_kernel<KPV>, gram64, k, rho, minv));
+  KP_SWITCH(kp, return launch_dependent(admm_minv_kernel<KPV>, dim3(1), 256, s, gram64, k, rho, minv));
   return cudaErrorInvalidValue;
 }
 
@@ -684,32 +675,15 @@ cudaError_t launch_prepare_tiles(const float *H, int64_t n, int k, int kp, void 
 }
 
 cudaError_t launch_reduce_iter(const ReduceArgs &a, int kp, cudaStream_t s) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(1 + (a.gram_part ? kp * kp / 16 : 0));
-  cfg.blockDim = dim3(256);
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  KP_SWITCH(kp, return cudaLaunchKernelEx(&cfg, reduce_iter_kernel<KPV>, a));
+  const dim3 grid(1 + (a.gram_part ? kp * kp / 16 : 0));
+  KP_SWITCH(kp, return launch_dependent(reduce_iter_kernel<KPV>, grid, 256, s, a));
   return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_gram_subset(const float *gram_part, int kp, const int *l1, int n1,
                                const int *l2, int n2, float *o1, float *o2, int kb, cudaStream_t s) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kp * kp / 16, 2);
-  cfg.blockDim = dim3(256);
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  KP_SWITCH(kp, return cudaLaunchKernelEx(&cfg, gram_subset_kernel<KPV>, gram_part, l1, n1, l2, n2,
-                                          o1, o2, kb));
+  KP_SWITCH(kp, return launch_dependent(gram_subset_kernel<KPV>, dim3(kp * kp / 16, 2), 256, s,
+                                        gram_part, l1, n1, l2, n2, o1, o2, kb));
   return cudaErrorInvalidValue;
 }
 

@@ -61,6 +61,7 @@ __device__ __forceinline__ void km_write_operand(const KmArgs &a, const float (*
 // operand D^-1 B: row i holds 1 / ||s_i|| in column labels_in[i]
 template <int KP>
 __global__ void __launch_bounds__(256) km_operand_kernel(KmArgs a) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __shared__ float Cs[kTileRows][KP + 1];
   const int64_t r0 = (int64_t)blockIdx.x * kTileRows;
   for (int e = threadIdx.x; e < kTileRows * (KP + 1); e += 256) (&Cs[0][0])[e] = 0.f;
@@ -116,6 +117,8 @@ __global__ void __launch_bounds__(256) km_centroid_kernel(KmArgs a) {
   __shared__ float Cs[kTileRows][KP + 1];
   __shared__ double part[G][KP];
   const int tile = blockIdx.x, tid = threadIdx.x;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   km_gather<KP>(a, Cs, tile);
   __syncthreads();
   const int c = tid % KP, g = tid / KP;
@@ -139,7 +142,9 @@ __global__ void __launch_bounds__(256) km_centroid_kernel(KmArgs a) {
 }
 
 // ||c_k||: 256 / KP threads per column, tiles g, g + G, ... each, the threads
-// in order; inv_norm = 0 for an empty cluster
+// in order; inv_norm = 0 for an empty cluster.  Runs beside the second product
+// (whose launch has seen the centroids complete) and waits for it before it
+// ends, as the assignment that follows needs both
 template <int KP>
 __global__ void __launch_bounds__(256) km_norms_kernel(KmArgs a) {
   constexpr int G = 256 / KP;
@@ -147,10 +152,11 @@ __global__ void __launch_bounds__(256) km_norms_kernel(KmArgs a) {
   const int c = threadIdx.x % KP, g = threadIdx.x / KP;
   double s = 0.0;
 #pragma unroll 4
-  for (int t = g; t < a.ntiles; t += G) s += a.colsq[(int64_t)t * KP + c];
+  for (int t = g; t < a.ntiles; t += G) s += __ldcg(a.colsq + (int64_t)t * KP + c);
   part[g][c] = s;
   __syncthreads();
   if (threadIdx.x >= KP) return;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   s = 0.0;
 #pragma unroll
   for (int i = 0; i < G; ++i) s += part[i][c];
@@ -166,6 +172,7 @@ __global__ void __launch_bounds__(256) km_assign_kernel(KmArgs a) {
   __shared__ float inv[KP];
   __shared__ double red[8];
   const int tile = blockIdx.x, r = threadIdx.x;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (r < KP) inv[r] = a.inv_norm[r];
   km_gather<KP>(a, Cs, tile);
   __syncthreads();
@@ -213,6 +220,7 @@ __global__ void __launch_bounds__(256) km_assign_kernel(KmArgs a) {
 __global__ void __launch_bounds__(256) km_final_kernel(KmArgs a) {
   __shared__ double red[2][8];
   const int tid = threadIdx.x;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int per = (a.ntiles + 255) / 256;
   double s0 = 0.0, s1 = 0.0;
   for (int t = tid * per; t < a.ntiles && t < (tid + 1) * per; ++t) {
@@ -270,17 +278,20 @@ cudaError_t launch_km_operand(const KmArgs &a, int kp, cudaStream_t s) {
 }
 
 cudaError_t launch_km_centroids(const KmArgs &a, int kp, cudaStream_t s) {
-  KM_KP_SWITCH(kp, {
-    km_centroid_kernel<KPV><<<a.ntiles, 256, 0, s>>>(a);
-    km_norms_kernel<KPV><<<1, 256, 0, s>>>(a);
-  });
-  return cudaGetLastError();
+  KM_KP_SWITCH(kp, return launch_dependent(km_centroid_kernel<KPV>, dim3(a.ntiles), 256, s, a));
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_km_norms(const KmArgs &a, int kp, cudaStream_t s) {
+  KM_KP_SWITCH(kp, return launch_dependent(km_norms_kernel<KPV>, dim3(1), 256, s, a));
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_km_assign(const KmArgs &a, int kp, cudaStream_t s) {
-  KM_KP_SWITCH(kp, km_assign_kernel<KPV><<<a.ntiles, 256, 0, s>>>(a));
-  km_final_kernel<<<1, 256, 0, s>>>(a);
-  return cudaGetLastError();
+  cudaError_t e = cudaErrorInvalidValue;
+  KM_KP_SWITCH(kp, e = launch_dependent(km_assign_kernel<KPV>, dim3(a.ntiles), 256, s, a));
+  if (e != cudaSuccess) return e;
+  return launch_dependent(km_final_kernel, dim3(1), 256, s, a);
 }
 
 }  // namespace symnmf

@@ -1699,6 +1699,7 @@ __global__ void __launch_bounds__(Cfg<DT, KP>::THREADS, 1)
   const int b = blockIdx.x;
   const Segs sg = cta_segments(a, b);
   int issued = 0;
+  if (a.chain & CHAIN_AFTER) asm volatile("griddepcontrol.wait;" ::: "memory");
   // a CTA takes all registers of its SM, so the next launch's CTAs start one
   // by one as this one's leave, or on SMs that this grid does not use
   if (a.chain & CHAIN_HEAD) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -1843,7 +1844,7 @@ cudaError_t launch_cfg(const ProdArgs &p, const EpiArgs &e, cudaStream_t s, cons
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = ta.fused || (ta.chain & CHAIN_NEXT) ? 1 : 0;
+  cfg.numAttrs = ta.fused || (ta.chain & (CHAIN_NEXT | CHAIN_AFTER)) ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, step_tc_kernel<DT, KP>, mS, mB, mB2, ta, e);
 }
 

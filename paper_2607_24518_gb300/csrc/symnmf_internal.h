@@ -88,6 +88,7 @@ struct ProdArgs {
 enum Chain {
   CHAIN_HEAD = 1,  // the next launch may start as this one's CTAs leave their SMs
   CHAIN_NEXT = 2,  // launched so: waits for the launch before it only before it ends
+  CHAIN_AFTER = 4,  // launched so: sets up, then waits for the launch before it
 };
 
 // Partial-sum layout of a product launch: split layout (SIMT: nsplit
@@ -251,6 +252,7 @@ cudaError_t launch_row_norms(const void *S, int64_t n, int64_t lds, int dtype, c
 cudaError_t launch_km_operand(const KmArgs &a, int kp, cudaStream_t s);
 // operand C from the partials of S (D^-1 B), and its column norms
 cudaError_t launch_km_centroids(const KmArgs &a, int kp, cudaStream_t s);
+cudaError_t launch_km_norms(const KmArgs &a, int kp, cudaStream_t s);
 // labels from the partials of S C, J and the changed count into out
 cudaError_t launch_km_assign(const KmArgs &a, int kp, cudaStream_t s);
 
