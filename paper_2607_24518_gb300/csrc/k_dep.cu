@@ -106,7 +106,11 @@ __global__ void __launch_bounds__(32 * kPrepY, 2)
         l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(u, b)), __fsub_rn(v, b)));
         h = u;
       }
-      m += (double)h + (double)l;
+      if (isfinite(h + l)) {
+        m += (double)h + (double)l;
+      } else {  // levels from about FLT_MAX / 64 overflow the run's high part
+        for (int64_t tt = t; tt < min(T, t + kRun); tt += kPrepY) m += (double)__ldg(col + tt * ldy);
+      }
     }
     m = total(m);
     if (y == 0) mean[x] = (float)(m / (double)T);

@@ -55,6 +55,27 @@ def test_columns_of_any_magnitude(L, center):
     assert np.array_equal(got, got.T)
 
 
+@pytest.mark.parametrize("T", [3, 64, 1100])
+def test_columns_of_a_level_whose_sum_leaves_fp32(L, T):
+    """Means are FP64 sums: a column at 1e37 or 3e38 has a finite mean although
+    64 of its entries add up to more than FP32 holds.  (T = 3: at most one
+    entry a thread; 64: four; 1100: more than a run of 64.)"""
+    n = 70
+    rng = np.random.default_rng(T)
+    Y = rng.standard_normal((T, 4)) @ rng.random((4, n)) + rng.standard_normal((T, n))
+    level = np.array([1.0, 1e20, 5e36, 1e37, -1e37, 3e38, -3e38])[np.arange(n) % 7]
+    Y = (level * (1.0 + 0.02 * np.clip(Y, -5, 5))).astype(np.float32)
+    assert np.isfinite(Y).all()
+    S = torch.full((n, n), -1.0, device=DEV)
+    L.symnmf_build_dependence(torch.tensor(Y, device=DEV), T, n, n, 1, L.F32, S, n)
+    C = (Y - Y.astype(np.float64).mean(0).astype(np.float32)).astype(np.float64)  # centred in FP32
+    C /= np.sqrt((C * C).sum(0))
+    ref = np.minimum(1.0, np.abs(C.T @ C))
+    np.fill_diagonal(ref, 1.0)
+    got = S.double().cpu().numpy()
+    assert np.max(np.abs(got - ref)) <= tol(T)
+
+
 @pytest.mark.parametrize("out", ["f32", "bf16", "fp8"])
 @pytest.mark.parametrize("T,n", [(2, 128), (128, 256), (129, 257), (31, 2048), (33, 2049), (160, 4353)])
 def test_tile_list_and_mirrors(L, T, n, out):
