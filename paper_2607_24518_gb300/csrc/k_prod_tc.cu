@@ -277,7 +277,7 @@ __device__ __forceinline__ void hgram_tile(const float *Hs, const float *Gs, flo
   for (int i = 0; i < RP; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
 #pragma unroll 4
   for (int d = 0; d < KP; ++d) {
-    const float4 m = __ldg(reinterpret_cast<const float4 *>(Gs + d * KP) + cg);
+    const float4 m = reinterpret_cast<const float4 *>(Gs + d * KP)[cg];
 #pragma unroll
     for (int i = 0; i < RP; ++i) {
       const float h = Hs[(rg + i * RS) * (KP + 1) + d];
@@ -419,7 +419,7 @@ __device__ __forceinline__ void tile_prep(const EpiArgs &e, int tp, float *Hs, f
     const float4 *gr = reinterpret_cast<const float4 *>(Gs + d * KP + cb);
 #pragma unroll
     for (int c4 = 0; c4 < Own<KP>::HG / 4; ++c4) {
-      const float4 gv = __ldg(gr + c4);
+      const float4 gv = gr[c4];
       hg[4 * c4 + 0] = fmaf(hv, gv.x, hg[4 * c4 + 0]);
       hg[4 * c4 + 1] = fmaf(hv, gv.y, hg[4 * c4 + 1]);
       hg[4 * c4 + 2] = fmaf(hv, gv.z, hg[4 * c4 + 2]);
@@ -804,8 +804,10 @@ __device__ void epilogue_role(const TcArgs &a, const EpiArgs &e, uint32_t tmem_b
   }
   // the Gram of H_t and the tile slots belong to the preceding reduction
   // kernel, which may still run (programmatic dependent launch).  The Gram
-  // is read from global memory: its next writer is the reduction kernel
-  // that follows this step, which starts only after this grid completes.
+  // is read from global memory by ordinary loads: it is written within this
+  // grid's lifetime, which the read-only path (__ldg) does not allow for.
+  // Its next writer is the reduction kernel that follows this step, which
+  // starts only after this grid completes.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const float *Gs = e.gram;
   constexpr int KH = Own<KP>::KH;
@@ -1152,7 +1154,9 @@ __device__ void folder_role(const TcArgs &a, uint32_t tmem_base, uint8_t *smem, 
     const int tp = (int)(u / a.n_cols), ci = unit_col(a, u);
     const int rt = a.row_list ? a.row_list[tp] : tp;
     const int ct = a.col_list ? a.col_list[ci] : ci;
-    return __ldg(a.sS + (int64_t)rt * a.ld_sS + ct) * __ldg(a.deq + ct);
+    // (the factors may be written while this CTA is set up, by the launch it
+    // waits for: never through the read-only path)
+    return __ldg(a.sS + (int64_t)rt * a.ld_sS + ct) * __ldcg(a.deq + ct);
   };
   // where the folders set the pace a whole-warp test first is quicker (n =
   // 20000: FP32 k = 32 271 -> 266 us, FP8 k = 64 118 -> 113); FP8 below kp = 64

@@ -196,3 +196,30 @@ def test_kmeans_fp8_storage(L):
     rows = np.arange(n)
     assert np.all(cos[rows, got] >= cos[rows, ref] - 2.0 ** -6)
     assert abs(Jt[0] - J) <= 2.0 ** -6 * n
+
+
+@pytest.mark.parametrize("n,Kc", [(1024, 16), (2300, 64), (500, 5)])
+def test_kmeans_fp8_iterations_equal_one_iteration_calls(L, n, Kc):
+    """The FP8 product reads the tile factors of its operand, which the small
+    kernel launched just before it writes anew in every iteration: six
+    iterations of one call give the labels and J of six calls of one
+    iteration, each of which starts with nothing in flight."""
+    S_t, _ = _tpdm(n, Kc, seed=n)
+    nt, lds = -(-n // 128), -(-n // 16) * 16
+    q = torch.zeros(n, lds, dtype=torch.uint8, device=DEV)
+    sc = torch.zeros(nt, nt, device=DEV)
+    L.symnmf_quantize_fp8(S_t, L.F32, n, n, n, q, lds, sc, nt, None)
+    h = L.symnmf_create_ld(q, n, lds, Kc, L.FP8E4M3)
+    try:
+        L.symnmf_set_tile_scales(h, sc, nt)
+        lab = _labels(n, Kc, seed=n + 1)
+        got, st, Jt = _run(L, h, lab, n, 6, tol=0.0)
+        one, J1 = lab, []
+        for _ in range(st.iters):
+            torch.cuda.synchronize()
+            out, _, J = _run(L, h, one.astype(np.int32), n, 1)
+            one = out
+            J1.append(J[0])
+    finally:
+        L.symnmf_destroy(h)
+    assert np.array_equal(got, one) and list(Jt) == J1
