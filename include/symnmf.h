@@ -243,8 +243,13 @@ int symnmf_step(symnmf_t h, const symnmf_hparams *hp, int32_t iters, symnmf_stat
 /* Step count handles together: each iteration of every live handle is
  * launched on the handle's own stream before any of them is checked, so
  * the handles' kernels overlap on the GPU; one host loop.  hps and
- * outs are arrays of count (outs may be NULL).  Returns the first error, or
- * SYMNMF_OK; per-handle convergence is in outs[i].converged. */
+ * outs are arrays of count (outs may be NULL).  A handle that has converged
+ * or failed runs no further iterations.  The grid of a small matrix depends
+ * on the row tiles of all handles still running, and with it the order of
+ * its FP32 partial sums: a handle's result is the same from run to run in the
+ * same company, and agrees with symnmf_step on it alone to FP32 rounding.
+ * Returns the first error, or SYMNMF_OK; per-handle convergence is in
+ * outs[i].converged. */
 int symnmf_batch_step(symnmf_t *hs, int32_t count, const symnmf_hparams *hps, int32_t iters,
                       symnmf_stats *outs);
 /* Cap the CTAs of the handle's tensor-core launches (0 = one per SM, the

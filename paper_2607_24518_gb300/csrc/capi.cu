@@ -1570,11 +1570,20 @@ int symnmf_batch_step(symnmf_t *hs, int32_t count, const symnmf_hparams *hps, in
       if (!first_err) first_err = rc;
     }
   }
-  int64_t tiles = 0;
-  for (int32_t i = 0; i < count; ++i) tiles += live[i] ? hs[i]->ntiles : 0;
-  for (int32_t i = 0; i < count; ++i)
-    if (live[i]) hs[i]->batch_tiles = (int)std::min<int64_t>(tiles, INT32_MAX);
+  // the tiles that share the SMs, counted anew whenever a handle leaves, so
+  // that the ones left get back the grids they would have without it
+  int32_t counted = -1;
+  auto share = [&]() {
+    const int32_t now = (int32_t)std::count(live.begin(), live.end(), 1);
+    if (now == counted) return;
+    counted = now;
+    int64_t tiles = 0;
+    for (int32_t i = 0; i < count; ++i) tiles += live[i] ? hs[i]->ntiles : 0;
+    for (int32_t i = 0; i < count; ++i)
+      if (hs[i]) hs[i]->batch_tiles = live[i] ? (int)std::min<int64_t>(tiles, INT32_MAX) : 0;
+  };
   for (int32_t it = 0; it < iters; ++it) {
+    share();
     // every live handle's iteration is launched before any check waits, so
     // one handle's check does not hold back the others' launches
     for (int32_t i = 0; i < count; ++i) {
@@ -1600,9 +1609,10 @@ int symnmf_batch_step(symnmf_t *hs, int32_t count, const symnmf_hparams *hps, in
     }
     if (!any) break;
   }
+  for (int32_t i = 0; i < count; ++i)
+    if (hs[i]) hs[i]->batch_tiles = 0;
   for (int32_t i = 0; i < count; ++i) {
     if (!hs[i]) continue;
-    hs[i]->batch_tiles = 0;
     if (!hs[i]->bad) {
       symnmf_t h = hs[i];
       const int64_t upto = h->ctrl.converged ? h->ctrl.t + 1 : h->ctrl.t;
