@@ -60,7 +60,7 @@ def test_columns_of_a_level_whose_sum_leaves_fp32(L, T):
     """Means are FP64 sums: a column at 1e37 or 3e38 has a finite mean although
     64 of its entries add up to more than FP32 holds.  (T = 3: at most one
     entry a thread; 64: four; 1100: more than a run of 64.)"""
-    n = 70
+    n = 72
     rng = np.random.default_rng(T)
     Y = rng.standard_normal((T, 4)) @ rng.random((4, n)) + rng.standard_normal((T, n))
     level = np.array([1.0, 1e20, 5e36, 1e37, -1e37, 3e38, -3e38])[np.arange(n) % 7]
