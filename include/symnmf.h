@@ -145,8 +145,9 @@ typedef struct symnmf_stats {
 /* ---------------------------------------------------------------- handles */
 
 /* Create a handle for S (device, n x n, row pitch n elements, dtype) and
- * rank k.  Computes ||S||_F^2 in FP64 (a single streaming pass; for FP8 at
- * symnmf_set_tile_scales).  Returns INVALID for n < 1 or null S/out,
+ * rank k.  Computes ||S||_F^2 to FP64 accuracy (a single streaming pass; runs of
+ * 64 entries in three FP32 words, exact words for FP8, joined in FP64; for FP8
+ * at symnmf_set_tile_scales).  Returns INVALID for n < 1 or null S/out,
  * UNSUPPORTED for k outside 1..64. */
 int symnmf_create(const void *S, int64_t n, int32_t k, int32_t dtype, symnmf_t *out);
 /* As symnmf_create with an explicit row pitch lds >= n (elements).  The
@@ -172,8 +173,8 @@ int symnmf_set_tile_scales(symnmf_t h, const float *scales, int64_t ld_scales);
  * pitch ld_src elements.  Outputs (device, caller-owned): q, rows x cols
  * bytes with row pitch ldq; scales, ceil(rows/128) x ceil(cols/128) FP32
  * with row pitch ld_scales; tile_sumsq (may be NULL), the FP64 sum of
- * squares of each unquantised tile in the layout of scales (for
- * symnmf_set_norm).  Tiles start at the band's first row and column, so a
+ * squares of each unquantised tile (to FP64 accuracy, as ||S||_F^2 of a handle)
+ * in the layout of scales (for symnmf_set_norm).  Tiles start at the band's first row and column, so a
  * band of a larger S must start at a multiple of 128 rows.  Asynchronous on
  * stream (cudaStream_t as void*, NULL = legacy default stream).  INVALID for
  * null q/src/scales, rows or cols < 1, a pitch below its width or another
@@ -430,7 +431,7 @@ int symnmf_set_matrix(symnmf_t h, const void *S, int64_t lds, const float *scale
  * Arithmetic: the centred values are FP32; G is formed on the tensor cores
  * from FP16 hi / lo pieces of each value, scaled by a power of two per column
  * (22 bits; hi hi + hi lo + lo hi, FP32 accumulation), about FP32 accuracy;
- * column norms are FP64.  A column with
+ * column means and norms have FP64 accuracy.  A column with
  * zero variance gives a zero row and column in S except S_ii = 1.
  * Scratch: n (4 T' + 4) bytes and 8 per SM of stream-ordered device memory
  * (T' = T rounded up to 32), freed before return.
@@ -487,8 +488,8 @@ typedef struct {
  * tol = 1e-4), or after max_iter iterations.
  * One iteration is two passes of the streamed product (S symmetric):
  * C = S (D^-1 B) with D = diag ||s_i|| and B the one-hot labels, then
- * P = S C, with cos_ik = P_ik / (||s_i|| ||c_k||); FP32 products, FP64
- * norms and FP64 fixed-order cross-tile sums, so runs are bit-reproducible.
+ * P = S C, with cos_ik = P_ik / (||s_i|| ||c_k||); FP32 products, norms of
+ * FP64 accuracy and FP64 fixed-order cross-tile sums, so runs are bit-reproducible.
  * Arguments: labels0 (device, n int32, entries in 0..K-1; an entry outside
  * that range puts its row in no cluster for the first iteration), labels
  * (device, n int32, written: the final labels), max_iter >= 1, tol >= 0,
@@ -498,7 +499,7 @@ typedef struct {
  * solver state (H, its MMA copy, the Gram, the optimizer buffers) is not
  * touched; the call synchronises the handle's stream once per iteration.
  * Errors: INVALID for null labels, max_iter < 1 or tol < 0 or NaN; OOM when
- * the scratch (n (8 + 8) + ceil(n/128) (16 + 8 kp) bytes) cannot be
+ * the scratch (n (12 + 8) + ceil(n/128) (16 + 8 kp) bytes) cannot be
  * allocated; CUDA / STATE as for symnmf_step. */
 int symnmf_spkmeans(symnmf_t h, const int32_t *labels0, int32_t *labels, int32_t max_iter,
                     double tol, double *J_trace, symnmf_kmeans_stats *stats);

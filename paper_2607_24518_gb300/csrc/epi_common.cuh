@@ -144,30 +144,69 @@ __device__ __forceinline__ void ff_xor_add(float &hi, float &lo, int o) {
   lo = __fsub_rn(t, __fsub_rn(hi, s));
 }
 
-// Running sum of squares as a float-float pair: the product is split exactly
-// by an FMA and the high parts are added by Knuth's TwoSum, so only the low
-// part (near 2^-23 of the sum) is rounded.  FP64 runs at two operations per
-// SM and cycle on this part; a run of 64 entries summed this way (rounding
-// near 2^-47) takes three FP64 operations instead of 128 and more.
-struct SqRun {
-  float h = 0.f, l = 0.f, m = 0.f;  // sum = h + l, m = largest magnitude
-  // SHORT: v has at most 12 significant bits, so its square is exact
-  template <bool SHORT = false>
-  __device__ __forceinline__ void add(float v) {
+// Running sum of squares of FP32 values with FP64 accuracy and few FP64
+// operations (two per SM and cycle on this part): a run of up to 64 values in
+// three FP32 words, joined in FP64 by flush().  With |v| <= cap (a power of
+// two) the words start at anchors, H at A = 64 cap^2 and L at 1.5 * 2^-16 A.
+// p = v^2 is below A / 64, so H stays in [A, 2 A), is never smaller than what
+// is added and Fast2Sum (Dekker 1971) gives the exact error of H + p in two
+// operations; that error and the product's own (one FMA) are at most 2^-24 A
+// and go into L in the same way, 2^-18 A in all; what L rounds off is at most
+// 2^-40 A each time and is added up in T.  Only those additions round, 2^-51 A
+// for a run at the very most.  ||S||^2 of uniform FP32 entries, n = 2048: off by
+// at most 2e-16 of itself (FP64 per entry 7e-16; two words without the third
+// 5e-15).  A larger value flushes and raises cap; what leaves [2^-40, 2^56],
+// where squares would lose bits or overflow, is summed in FP64.  EXACT: v has at
+// most 12 significant bits, so p is exact.
+template <bool EXACT = false>
+struct SqSum {
+  float H = 0.f, L = 0.f, T = 0.f, cap = 0.f;
+  double acc = 0.0;  // the sum, once flushed
+  __device__ __forceinline__ static float hi(float c) { return 64.f * c * c; }
+  __device__ __forceinline__ static float lo(float c) { return 0x1.8p-10f * c * c; }
+  __device__ __forceinline__ void put(float v) {
     const float p = __fmul_rn(v, v);
-    const float t = __fadd_rn(h, p), b = __fsub_rn(t, h);
-    float e = __fadd_rn(__fsub_rn(h, __fsub_rn(t, b)), __fsub_rn(p, b));
-    if constexpr (!SHORT) e = __fadd_rn(e, fmaf(v, v, -p));
-    l = __fadd_rn(l, e);
-    h = t;
-    m = fmaxf(m, fabsf(v));
+    const float t = __fadd_rn(H, p), e = __fsub_rn(p, __fsub_rn(t, H));
+    H = t;
+    low(e);
+    if constexpr (!EXACT) low(fmaf(v, v, -p));
   }
-  // squares that neither overflow nor lose bits to underflow; otherwise the
-  // caller sums the run in FP64
-  __device__ __forceinline__ bool in_range() const {
-    return m < 0x1p56f && (m == 0.f || m > 0x1p-40f);
+  __device__ __forceinline__ void low(float e) {
+    const float t = __fadd_rn(L, e);
+    T = __fadd_rn(T, __fsub_rn(e, __fsub_rn(t, L)));
+    L = t;
   }
-  __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+  // H - A and L - 1.5 * 2^-16 A are exact; after at most 64 values
+  __device__ __forceinline__ void flush() {
+    acc += (double)__fsub_rn(H, hi(cap));
+    acc += (double)__fsub_rn(L, lo(cap));
+    acc += (double)T;
+    H = hi(cap);
+    L = lo(cap);
+    T = 0.f;
+  }
+  // ready for values up to m (m > cap); false: they have to be summed in FP64
+  __device__ __forceinline__ bool raise(float m) {
+    if (!(m > 0x1p-40f && m < 0x1p56f)) return false;
+    if (H != 0.f) flush();  // (nothing but zeros before)
+    cap = __uint_as_float((__float_as_uint(m) & 0x7F800000u) + 0x00800000u);
+    H = hi(cap);
+    L = lo(cap);
+    return true;
+  }
+  template <int N>
+  __device__ __forceinline__ void add(const float (&v)[N]) {
+    float m = 0.f;
+#pragma unroll
+    for (int i = 0; i < N; ++i) m = fmaxf(m, fabsf(v[i]));
+    if (m > cap && !raise(m)) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) acc = fma((double)v[i], (double)v[i], acc);
+      return;
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) put(v[i]);
+  }
 };
 
 // entry i of S (FP8: the code's value, without its tile scale)
@@ -177,14 +216,37 @@ __device__ __forceinline__ float s_entry(const void *S, int64_t i) {
   else if constexpr (DT == 1) return bf16_val(__ldg(reinterpret_cast<const uint16_t *>(S) + i));
   else return e4m3_val(__ldg(reinterpret_cast<const uint8_t *>(S) + i));
 }
-// a lane's 16 entries of columns c0 .. c0 + 511 of a row of S, in 16-byte
-// groups one warp apart (vec: every row starts on a 16-byte boundary), else
-// element by element; entries from column n on are 0.  FP8: the 16 entries
-// are consecutive, so they share a tile scale.
+// 16 E4M3 codes of a row from column c on (vec: the row starts on a 16-byte
+// boundary, c is a multiple of 16), 0 from column n on; and their values
+__device__ __forceinline__ uint4 load_codes(const void *S, int64_t rowbase, int64_t c, int64_t n,
+                                            bool vec) {
+  const uint8_t *p = reinterpret_cast<const uint8_t *>(S) + rowbase + c;
+  if (vec && c + 16 <= n) return __ldg(reinterpret_cast<const uint4 *>(p));
+  uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int j = 0; j < 16; ++j)
+    if (c + j < n) w[j / 4] |= (uint32_t)__ldg(p + j) << (8 * (j % 4));
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+__device__ __forceinline__ void e4m3_vals(const uint4 &x, float (&v)[16]) {
+  const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const float2 f = __half22float2(__half2(__nv_cvt_fp8x2_to_halfraw2(
+          (__nv_fp8x2_storage_t)(w[j] >> (16 * u)), __NV_E4M3)));
+      v[4 * j + 2 * u] = f.x;
+      v[4 * j + 2 * u + 1] = f.y;
+    }
+}
+// a lane's 16 entries of columns c0 .. c0 + 511 of a row of S (FP32, BF16), in
+// 16-byte groups one warp apart (vec: every row starts on a 16-byte boundary),
+// else element by element; entries from column n on are 0
 template <int DT>
 __device__ __forceinline__ void load16(const void *S, int64_t rowbase, int64_t c0, int64_t n,
                                        bool vec, int lane, float (&v)[16]) {
-  constexpr int W = DT == 0 ? 4 : DT == 1 ? 8 : 16;  // entries of a 16-byte group
+  constexpr int W = DT == 0 ? 4 : 8;  // entries of a 16-byte group
 #pragma unroll
   for (int i = 0; i < 16 / W; ++i) {
     const int64_t c = c0 + (i * 32 + lane) * W;
@@ -196,17 +258,9 @@ __device__ __forceinline__ void load16(const void *S, int64_t rowbase, int64_t c
       for (int j = 0; j < 4; ++j) {
         if constexpr (DT == 0) {
           v[4 * i + j] = __uint_as_float(w[j]);
-        } else if constexpr (DT == 1) {
+        } else {
           v[8 * i + 2 * j] = __uint_as_float(w[j] << 16);
           v[8 * i + 2 * j + 1] = __uint_as_float(w[j] & 0xFFFF0000u);
-        } else {
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const float2 f = __half22float2(__half2(__nv_cvt_fp8x2_to_halfraw2(
-                (__nv_fp8x2_storage_t)(w[j] >> (16 * u)), __NV_E4M3)));
-            v[4 * j + 2 * u] = f.x;
-            v[4 * j + 2 * u + 1] = f.y;
-          }
         }
       }
     } else {
@@ -216,51 +270,77 @@ __device__ __forceinline__ void load16(const void *S, int64_t rowbase, int64_t c
   }
 }
 
-// the lane's entries of columns [c0, c1) (as load16 deals them) summed in FP64
-template <int DT>
-__device__ __noinline__ double row_sumsq_lane64(const void *S, int64_t rowbase, int64_t c0,
-                                                int64_t c1, int64_t n, const float *scales,
-                                                int lane) {
-  constexpr int W = DT == 0 ? 4 : DT == 1 ? 8 : 16;
-  double acc = 0.0;
-  for (int64_t c = c0 + lane * W; c < c1; c += 32 * W)
-    for (int j = 0; j < W && c + j < n; ++j) {
-      double x = (double)s_entry<DT>(S, rowbase + c + j);
-      if constexpr (DT == 2) x *= (double)scales[(c + j) / kTileRows];
-      acc = fma(x, x, acc);
-    }
-  return acc;
-}
-
-// One lane's share of sum_j S_rj^2 over row r: runs of 64 entries in
-// float-float form, the runs in FP64.  FP8: a power-of-two tile scale (all
-// that symnmf_quantize_fp8 writes) is exact in FP32; other scales and values
-// out of SqRun's range take the FP64 sum.  `scales`: the row's tile scales.
+// One lane's share of sum_j S_rj^2 over row r, in runs of 64 entries.  FP8: a
+// code's square has at most 8 significant bits, none below 2^-18, and 64 of
+// them stay below 2^24, so with H from 2^24 on (ulp 2) and L (at most one per
+// code, multiples of 2^-18) a run is exact in two words and four operations per
+// code; the tile scale enters in FP64, whenever it changes (`scales`: the row's
+// tile scales).  n = 12000, ||S||^2: FP32 111, BF16 106, FP8 48 us (two words,
+// which hold 48 bits: 100, 105 and 72, and 1220 with scales that are no powers
+// of two; FP64 per entry: 555, 556 and 1068).
 template <int DT>
 __device__ __forceinline__ double row_sumsq_lane(const void *S, int64_t rowbase, int64_t n,
                                                  const float *scales, bool vec, int lane) {
-  double acc = 0.0;
-  for (int64_t c0 = 0; c0 < n; c0 += 2048) {
-    SqRun s;
-    bool exact = true;
-    // loads in flight per lane: one chunk of FP32 is four, of FP8 one
-#pragma unroll (DT == 0 ? 1 : DT == 1 ? 2 : 4)
-    for (int i = 0; i < 4; ++i) {
-      const int64_t cc = c0 + 512 * i;
-      if (DT != 2 && cc >= n) break;
-      float v[16], sc = 1.f;
-      load16<DT>(S, rowbase, cc, n, vec, lane, v);
-      if constexpr (DT == 2) {
-        sc = __ldg(scales + min(cc + 16 * lane, n - 1) / kTileRows);
-        exact = exact && (__float_as_uint(sc) & 0x7FFFFFu) == 0u;
-      }
+  if constexpr (DT == 2) {
+    double acc = 0.0, s2 = 1.0;
+    float H = 0x1p24f, L = 0.f, scale = 1.f;
+    auto flush = [&]() {
+      acc = fma(s2, (double)__fsub_rn(H, 0x1p24f) + (double)L, acc);
+      H = 0x1p24f;
+      L = 0.f;
+    };
+    auto add = [&](const uint4 &x) {
+      float v[16];
+      e4m3_vals(x, v);
 #pragma unroll
-      for (int j = 0; j < 16; ++j) s.template add<(DT == 2)>(DT == 2 ? v[j] * sc : v[j]);
+      for (int j = 0; j < 16; ++j) {
+        const float t = fmaf(v[j], v[j], H);
+        L = __fadd_rn(L, fmaf(v[j], v[j], -__fsub_rn(t, H)));
+        H = t;
+      }
+    };
+    for (int64_t c0 = 16 * lane; c0 < n + 16 * lane; c0 += 2048) {
+      uint4 x[4];
+      float sc[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {  // all loads of a run first
+        const int64_t c = c0 + 512 * i;
+        x[i] = load_codes(S, rowbase, c, n, vec);
+        sc[i] = __ldg(scales + min(c, n - 1) / kTileRows);
+      }
+      if (sc[0] == scale && sc[1] == scale && sc[2] == scale && sc[3] == scale) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) add(x[i]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (sc[i] != scale) {
+            flush();
+            scale = sc[i];
+            s2 = (double)scale * (double)scale;
+          }
+          add(x[i]);
+        }
+      }
+      flush();
     }
-    if (exact && s.in_range()) acc += s.value();
-    else acc += row_sumsq_lane64<DT>(S, rowbase, c0, min(c0 + 2048, n), n, scales, lane);
+    return acc;
+  } else {
+    SqSum<(DT == 1)> s;
+    for (int64_t c0 = 0; c0 < n; c0 += 2048) {
+      // loads in flight per lane: one chunk of FP32 is four, of BF16 two
+#pragma unroll (DT == 0 ? 1 : 2)
+      for (int i = 0; i < 4; ++i) {
+        const int64_t cc = c0 + 512 * i;
+        if (cc >= n) break;
+        float v[16];
+        load16<DT>(S, rowbase, cc, n, vec, lane, v);
+        s.add(v);
+      }
+      s.flush();
+    }
+    return s.acc;
   }
-  return acc;
 }
 
 }  // namespace symnmf

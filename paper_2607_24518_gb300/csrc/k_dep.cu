@@ -65,10 +65,18 @@ constexpr size_t kDepSmem = 1024 + (size_t)kDepStages * kDepStage + 256 + 256 * 
 constexpr int kDepThreads = 320;  // warp 0 TMA, warp 1 MMA, warps 2-9 epilogue
 constexpr int kDepGroup = 16;     // row tiles that sweep the column blocks together
 
+// s += v; returns the exact error (Knuth's TwoSum)
+__device__ __forceinline__ float two_sum(float &s, float v) {
+  const float t = __fadd_rn(s, v), b = __fsub_rn(t, s);
+  const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b));
+  s = t;
+  return e;
+}
+
 // One CTA per 32 variables, 32 x 16 threads: thread (x, y) sums variable
 // i0 + x over the observations y, y + 16, ...  Runs of 64 observations are
-// float-float pairs (SqRun and TwoSum), the runs are added in FP64 and the 16
-// threads of a variable in order.  Bound by HBM once Y is read; FP64 per
+// kept in three FP32 words (TwoSum, SqSum), the runs are added in FP64 and the
+// 16 threads of a variable in order.  Bound by HBM once Y is read; FP64 per
 // entry in one thread per variable was bound by latency and the FP64 pipe.
 constexpr int kPrepY = 16;   // threads per variable
 constexpr int kPrepT = 128;  // observations transposed together
@@ -93,23 +101,26 @@ __global__ void __launch_bounds__(32 * kPrepY, 2)
     __syncthreads();
     return s;
   };
-  constexpr int64_t kRun = 64 * kPrepY;
+  // (T is at most 2^30)
+  constexpr int kRun = 64 * kPrepY;
+  const int Ti = (int)T;
+  const int64_t step = (int64_t)kPrepY * ldy;
   float mf = 0.f;
   if (center) {
     double m = 0.0;
-    for (int64_t t = y; t < T; t += kRun) {
-      float h = 0.f, l = 0.f;
+    for (int t = y; t < Ti; t += kRun) {
+      float h = 0.f, l = 0.f, r = 0.f;  // what h and l round off goes one word down
+      const float *p = col + t * ldy;
+      const int e = min(Ti, t + kRun);
 #pragma unroll 8
-      for (int64_t tt = t; tt < min(T, t + kRun); tt += kPrepY) {
-        const float v = __ldg(col + tt * ldy);
-        const float u = __fadd_rn(h, v), b = __fsub_rn(u, h);
-        l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(u, b)), __fsub_rn(v, b)));
-        h = u;
-      }
+      for (int tt = t; tt < e; tt += kPrepY, p += step) r = __fadd_rn(r, two_sum(l, two_sum(h, __ldg(p))));
       if (isfinite(h + l)) {
-        m += (double)h + (double)l;
-      } else {  // levels from about FLT_MAX / 64 overflow the run's high part
-        for (int64_t tt = t; tt < min(T, t + kRun); tt += kPrepY) m += (double)__ldg(col + tt * ldy);
+        m += (double)h;
+        m += (double)l;
+        m += (double)r;
+      } else {  // levels from about FLT_MAX / 64 overflow the run's high word
+        p = col + t * ldy;
+        for (int tt = t; tt < e; tt += kPrepY, p += step) m += (double)__ldg(p);
       }
     }
     m = total(m);
@@ -117,20 +128,18 @@ __global__ void __launch_bounds__(32 * kPrepY, 2)
     __syncthreads();
     mf = mean[x];
   }
-  double d = 0.0;
-  for (int64_t t = y; t < T; t += kRun) {
-    SqRun s;
-#pragma unroll 8
-    for (int64_t tt = t; tt < min(T, t + kRun); tt += kPrepY) s.add(__ldg(col + tt * ldy) - mf);
-    if (s.in_range()) {
-      d += s.value();
-    } else {
-      for (int64_t tt = t; tt < min(T, t + kRun); tt += kPrepY) {
-        const double c = (double)(__ldg(col + tt * ldy) - mf);
-        d = fma(c, c, d);
-      }
+  SqSum<> sq;
+  for (int t = y; t < Ti; t += kRun) {
+    const float *p = col + t * ldy;
+    for (int t8 = t; t8 < min(Ti, t + kRun); t8 += 8 * kPrepY) {
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u, p += step) v[u] = t8 + u * kPrepY < Ti ? __ldg(p) - mf : 0.f;
+      sq.add(v);
     }
+    sq.flush();
   }
+  double d = sq.acc;
   d = total(d);
   if (y == 0) {
     // s = 2^e with s sqrt(d) in [2^14, 2^15); 1 for a column without a norm

@@ -462,10 +462,11 @@ __global__ void __launch_bounds__(256) gram_subset_kernel(const float *gram_part
   (blockIdx.y == 0 ? o1 : o2)[e] = (float)s;
 }
 
-// ||S||_F^2: one warp per row, runs of 64 entries as float-float sums, runs
-// and rows in FP64.  Bound by HBM; a conversion and a multiply-add per entry
-// in FP64 bounded it by the FP64 pipe before (n=12000 FP8: 1072 -> 74 us,
-// 1.9 TB/s).
+// ||S||_F^2: one warp per row, runs of 64 entries in FP32 words (row_sumsq_lane),
+// runs and rows in FP64.  FP32 is bound by HBM (n = 12000: 111 us, 5.2 TB/s),
+// BF16 and FP8 by the operations per entry (106 and 48 us); a conversion and a
+// multiply-add per entry in FP64 bounded all of them by the FP64 pipe (555 to
+// 1068 us).
 template <int DT>
 __global__ void __launch_bounds__(256, 4) norm_s2_kernel(const void *S, int64_t n, int64_t lds,
                                                       const float *scales, int64_t ld_scales,

@@ -28,7 +28,7 @@
 namespace symnmf {
 namespace {
 
-// ||s_i|| in FP64: one warp per row, runs of 64 entries as float-float sums
+// ||s_i|| in FP64: one warp per row, runs of 64 entries in FP32 words (SqSum)
 template <int DT>
 __global__ void __launch_bounds__(256, 4) row_norms_kernel(const void *S, int64_t n, int64_t lds,
                                                         const float *scales, int64_t ld_scales,
@@ -109,7 +109,7 @@ __device__ __forceinline__ void km_gather(const KmArgs &a, float (*Cs)[KP + 1], 
 }
 
 // centroid rows C_I = sum of the partials, and per-tile column sums of
-// squares: 256 / KP threads per column, each a float-float run of its rows,
+// squares: 256 / KP threads per column, each a run (SqSum) of its rows,
 // added in order in FP64
 template <int KP>
 __global__ void __launch_bounds__(256) km_centroid_kernel(KmArgs a) {
@@ -122,12 +122,17 @@ __global__ void __launch_bounds__(256) km_centroid_kernel(KmArgs a) {
   km_gather<KP>(a, Cs, tile);
   __syncthreads();
   const int c = tid % KP, g = tid / KP;
-  SqRun s;
+  float m = 0.f;
 #pragma unroll 8
-  for (int r = g * RG; r < (g + 1) * RG; ++r) s.add(Cs[r][c]);
-  double d = s.value();
-  if (!s.in_range()) {
-    d = 0.0;
+  for (int r = g * RG; r < (g + 1) * RG; ++r) m = fmaxf(m, fabsf(Cs[r][c]));
+  SqSum<> s;
+  double d = 0.0;
+  if (m == 0.f || s.raise(m)) {
+#pragma unroll 8
+    for (int r = g * RG; r < (g + 1) * RG; ++r) s.put(Cs[r][c]);
+    s.flush();
+    d = s.acc;
+  } else {
     for (int r = g * RG; r < (g + 1) * RG; ++r) d = fma((double)Cs[r][c], (double)Cs[r][c], d);
   }
   part[g][c] = d;

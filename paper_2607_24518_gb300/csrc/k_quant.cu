@@ -14,9 +14,10 @@ namespace {
 
 // 256 threads: warp w covers rows 16 w .. 16 w + 15, lane l columns 4 l .. 4 l + 3.
 // Bound by HBM (source read once, codes written once).  The sum of squares
-// runs in float-float form over the thread's 64 entries (FP64 per entry bounded the kernel
-// by the FP64 pipe; n=12000 FP32: 626 -> 162 us, 4.4 TB/s); vsrc / vdst: 4-entry loads and 4-code stores,
-// when base and pitch are aligned to them.
+// of the thread's 64 entries is kept in FP32 words with FP64 accuracy (SqSum;
+// FP64 per entry bounded the kernel by the FP64 pipe; n=12000 FP32: 626 -> 182
+// us); vsrc / vdst: 4-entry loads and 4-code stores, when base and pitch are
+// aligned to them.
 template <int SRC>
 __global__ void __launch_bounds__(256) quantize_kernel(const void *src, int64_t rows, int64_t cols,
                                                        int64_t ld_src, uint8_t *q, int64_t ldq,
@@ -28,7 +29,6 @@ __global__ void __launch_bounds__(256) quantize_kernel(const void *src, int64_t 
   const int64_t r0 = (int64_t)blockIdx.y * kTileRows, c0 = (int64_t)blockIdx.x * kTileRows;
   const int64_t c = c0 + lane * 4;
   float v[16][4];
-  float m = 0.f;
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
     const int64_t r = r0 + warp * 16 + i;
@@ -52,27 +52,27 @@ __global__ void __launch_bounds__(256) quantize_kernel(const void *src, int64_t 
       for (int j = 0; j < 4; ++j) v[i][j] = (r < rows && c + j < cols) ? s_entry<SRC>(src, at + j) : 0.f;
     }
   }
+  float m = 0.f;
+#pragma unroll
+  for (int i = 0; i < 16; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) m = fmaxf(m, fabsf(v[i][j]));
   double ss = 0.0;
   if (tile_sumsq) {
-    SqRun s;
+    SqSum<SRC == 1> s;
+    if (m == 0.f || s.raise(m)) {
 #pragma unroll
-    for (int i = 0; i < 16; ++i)
+      for (int i = 0; i < 16; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) s.add(v[i][j]);
-    m = s.m;
-    if (s.in_range()) {
-      ss = s.value();
+        for (int j = 0; j < 4; ++j) s.put(v[i][j]);
+      s.flush();
+      ss = s.acc;
     } else {
 #pragma unroll
       for (int i = 0; i < 16; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) ss = fma((double)v[i][j], (double)v[i][j], ss);
     }
-  } else {
-#pragma unroll
-    for (int i = 0; i < 16; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) m = fmaxf(m, fabsf(v[i][j]));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));

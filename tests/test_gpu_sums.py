@@ -1,17 +1,21 @@
-"""Sums of squares of S in FP64 accuracy: ||S||^2 of a handle, the tile sums
-of the quantiser and the row norms of spherical K-means, at the edges of
-their 16-entry groups, 64-entry runs and 512-column chunks, for aligned and
-unaligned rows, and for values and tile scales that leave the float-float
-form for the FP64 sum.  Reference: numpy in FP64.  Bound: a run of 64 entries
-rounds its low part (2^-24 of the sum) 64 times, 64 * 2^-24 * 2^-23 = 2^-41;
-FP64 sums over n <= 2100 terms add less."""
+"""Sums of squares of S in FP64 accuracy: ||S||^2 of a handle and the tile sums
+of the quantiser, and through the objective of a Lloyd step the row norms of
+spherical K-means, at the edges of their 16-entry groups, 64-entry runs and
+512-column chunks, for aligned and unaligned rows, for values that leave the
+FP32 words for the FP64 sum and for tile scales that are no powers of two.
+Reference: numpy in FP64.  Bound: a run of 64 entries rounds only in its third
+word, 128 times at most 2^-58 of 64 cap^2 with cap at most twice the largest
+entry: 2^-43 of its square if every rounding were the worst and all went one
+way.  A run of uniform entries (their cubes) sums to 21 (9) such squares, so
+2^-46; one or two entries do not reach the third word, and FP64 sums over n <=
+2100 terms add less."""
 import numpy as np
 import pytest
 import torch
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
-REL = 2.0 ** -41
+REL = 2.0 ** -46
 
 
 @pytest.fixture(scope="module")
@@ -33,7 +37,7 @@ def test_norm_of_a_handle(L, n, pad, dtype, scale):
     if dtype == "fp8":
         nt = -(-n // 128)
         q = (S * 448).to(torch.float8_e4m3fn)
-        # powers of two, and one factor that is none (the FP64 path)
+        # powers of two, times a factor that is none for two of the three scales
         sc = torch.tensor(scale * 2.0 ** rng.integers(-8, 0, (nt, nt)), dtype=torch.float32, device=DEV)
         h = L.symnmf_create_ld(q.view(torch.uint8), n, lds, 4, L.FP8E4M3)
         L.symnmf_set_tile_scales(h, sc, nt)
@@ -48,6 +52,22 @@ def test_norm_of_a_handle(L, n, pad, dtype, scale):
         assert abs(L.symnmf_get_norm(h) - ref) <= REL * ref
     finally:
         L.symnmf_destroy(h)
+
+
+def test_norm_when_the_largest_entry_comes_last(L):
+    """Entries that grow along a row by 2^60 in all raise the bound of the runs
+    again and again; zeros and entries below 2^-40 come first."""
+    n = 700
+    rng = np.random.default_rng(5)
+    S = (rng.random((n, n)) * 2.0 ** np.linspace(-50, 10, n)[None, :]).astype(np.float32)
+    S[:, :40] = 0.0
+    for M in (S, S[:, ::-1].copy(), np.where(rng.random((n, n)) < 0.01, S, np.float32(0))):
+        h = L.symnmf_create(torch.tensor(M, device=DEV), n, 4, L.F32)
+        try:
+            ref = float(np.sum(M.astype(np.float64) ** 2))
+            assert abs(L.symnmf_get_norm(h) - ref) <= 2.0 ** -43 * ref
+        finally:
+            L.symnmf_destroy(h)
 
 
 @pytest.mark.parametrize("src", ["f32", "bf16"])
