@@ -144,6 +144,31 @@ __device__ __forceinline__ void ff_xor_add(float &hi, float &lo, int o) {
   lo = __fsub_rn(t, __fsub_rn(hi, s));
 }
 
+// Sum of x over the warp in FP64, every lane the same bits: the values as
+// 64-bit integers in units of 2^-34 of the largest one's last place, so that an
+// integer tree adds them exactly (24 + 34 bits and 5 for 32 lanes); what lies
+// below that unit, 2^-57 of the largest value, is cut off.  An integer tree
+// takes two shuffles and two additions a level, as many shuffles as and fewer
+// operations than float-float pairs, which hold 48 bits.  Infinities and NaN:
+// the FP32 sum.
+__device__ __forceinline__ double warp_sum64(float x) {
+  const uint32_t u = __float_as_uint(x), a = u & 0x7FFFFFFFu;
+  const uint32_t top = __reduce_max_sync(0xffffffffu, a);
+  if (top >= 0x7F800000u) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return (double)x;
+  }
+  // exponent fields, 1 for subnormals as for the smallest normal numbers
+  const int et = max((int)(top >> 23), 1), ex = max((int)(a >> 23), 1);
+  int64_t m = (int64_t)((a & 0x7FFFFFu) | (a >= 0x800000u ? 0x800000u : 0u)) << 34;
+  m = et - ex < 58 ? m >> (et - ex) : 0;
+  if (u >> 31) m = -m;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, (long long)m, o);
+  return (double)m * __hiloint2double((et - 150 - 34 + 1023) << 20, 0);
+}
+
 // Running sum of squares of FP32 values with FP64 accuracy and few FP64
 // operations (two per SM and cycle on this part): a run of up to 64 values in
 // three FP32 words, joined in FP64 by flush().  With |v| <= cap (a power of

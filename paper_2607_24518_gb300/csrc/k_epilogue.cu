@@ -112,9 +112,10 @@ __device__ __forceinline__ void parts_of(const float *P, int nsplit, int skG, in
 // shared-memory reads: the H Gram products are formed in 4-column register
 // blocks and the state moves in 16-byte rows.  Multiply-adds are written out,
 // so that every padded rank rounds the same way (restarts in one handle are
-// bit-equal to separate handles).  n = 50000, kp = 64, block mode 337 -> 95
-// us; n = 5001, kp = 32 33 -> 12; n = 3001, kp = 16 19 -> 9.6 (two shared
-// reads per FMA and FP64 block sums before).
+// bit-equal to separate handles).  n = 50000, kp = 64, block mode 337 -> 89
+// us; n = 5001, kp = 32 33 -> 11; n = 3001, kp = 16 19 -> 8.9 (two shared
+// reads per FMA and FP64 block sums before; exact warp sums instead of
+// float-float trees take 0.6 us off the last).
 template <int KP>
 __global__ void __launch_bounds__(EpiK<KP>::T, KP == 64 ? 1 : 1024 / EpiK<KP>::T)
     epilogue_kernel(EpiArgs a) {
@@ -305,18 +306,16 @@ __global__ void __launch_bounds__(EpiK<KP>::T, KP == 64 ? 1 : 1024 / EpiK<KP>::T
     __syncthreads();  // Hs holds the tile of H_{t+1}
     tile_tail<KP, T>(Hs, r0, a.Btn, a.bt_fmt, a.ldb, a.gram_part, tile);
   }
-  // tile scalars: warp xor trees in float-float form, warps in order in FP64
-  float fh[3] = {tr, kkt2, sumA}, fl[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-    for (int i = 0; i < 3; ++i) ff_xor_add(fh[i], fl[i], o);
+  // tile scalars: exact warp sums (FP64 trees would take 15 slow additions a
+  // lane), warps in order in FP64
+  const float sc[3] = {tr, kkt2, sumA};
   const unsigned nf = __reduce_add_sync(0xffffffffu, (unsigned)nonfin);
-  if ((tid & 31) == 0) {
 #pragma unroll
-    for (int i = 0; i < 3; ++i) red[tid >> 5][i] = (double)fh[i] + (double)fl[i];
-    red[tid >> 5][3] = (double)nf;
+  for (int i = 0; i < 3; ++i) {
+    const double v = warp_sum64(sc[i]);
+    if ((tid & 31) == 0) red[tid >> 5][i] = v;
   }
+  if ((tid & 31) == 0) red[tid >> 5][3] = (double)nf;
   __syncthreads();
   if (tid < 4 && a.slots) {
     double s = 0.0;

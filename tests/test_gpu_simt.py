@@ -89,3 +89,27 @@ def test_one_step_of_the_stand_alone_epilogue(L, n, k, method):
             assert np.linalg.norm(got.double().cpu().numpy() - ref) <= tol
     finally:
         L.symnmf_destroy(h)
+
+
+@pytest.mark.parametrize("n,k", [(129, 8), (300, 11), (257, 33), (400, 64)])
+def test_tile_scalars_of_the_stand_alone_epilogue_are_fp64_sums(L, n, k):
+    """With H = 0 the gradient is 0 and the accumulator stays as it is, so the
+    record's sum(G) is the sum of what was put there: 2^50 once per tile,
+    several 3 * 2^25 and many ones.  They need 51 bits, one thread holds one of
+    them at most (rows below 32 and every fourth column of a tile), and an FP64
+    sum of them is exact."""
+    h, _, _, keep = _handle(L, n, k, "f32", seed=n)
+    try:
+        L.symnmf_set_H(h, torch.zeros(n, k, device=DEV))
+        A = np.zeros((n, k), dtype=np.float32)
+        rng = np.random.default_rng(k)
+        for r0 in range(0, n, 128):
+            rows = min(32, n - r0)
+            v = rng.choice(np.array([1.0, 3 * 2.0 ** 25, 0.0]), size=(rows, -(-k // 4)))
+            v[rng.integers(rows), rng.integers(v.shape[1])] = 2.0 ** 50
+            A[r0:r0 + rows, ::4] = v
+        L.symnmf_set_buffer(h, L.BUF_ACC, torch.tensor(A, device=DEV))
+        L.symnmf_step(h, L.symnmf_hparams_default(L.ADAGRAD), 1)
+        assert L.symnmf_get_trace(h)[-1].sumA == float(A.astype(np.float64).sum())
+    finally:
+        L.symnmf_destroy(h)
