@@ -434,7 +434,7 @@ int prod(symnmf_t h, const int *row_list, int n_rows, const int *col_list, int n
   a.batch_tiles = h->batch_tiles;
   a.out = out;
   const int64_t most = std::min<int64_t>(64, h->pq_cap_tiles / std::max(1, n_rows));
-  const int ns = simt_shares(n_rows, n_cols, h->num_sms, (int)std::max<int64_t>(1, most));
+  const int ns = simt_shares(n_rows, n_cols, h->kp, h->num_sms, (int)std::max<int64_t>(1, most));
   a.nsplit = ns;
   lay->nsplit = ns;
   lay->skG = 0;

@@ -295,7 +295,7 @@ extern "C" int symnmf_objective_noalloc(const void *S, int64_t n, int64_t lds, i
   a.H = H;
   a.k = k;
   a.ntiles = (int)ntiles;
-  a.split = simt_split(a.ntiles, a.ntiles, 2 * sms, kSplit);
+  a.split = simt_split(a.ntiles, a.ntiles, kp, 2 * sms, kSplit, kSplit);
   a.normS2 = normS2;
   a.tr_part = reinterpret_cast<double *>(base);
   a.gram_part = reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(base) + tr_bytes);

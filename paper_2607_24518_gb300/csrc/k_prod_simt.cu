@@ -4,6 +4,8 @@
 // (S row pitch not a multiple of 16 bytes).  One CTA owns one 128-row tile
 // and a contiguous share (split) of the column-tile list; partial sums go
 // to out[split][row_pos] and are added in split order by the epilogue.
+#include <algorithm>
+
 #include "simt_tile.cuh"
 #include "symnmf_internal.h"
 
@@ -60,8 +62,10 @@ cudaError_t launch_prod_simt(const ProdArgs &a, cudaStream_t s) {
   }
 }
 
-int simt_shares(int rows, int cols, int num_sms, int most) {
-  return simt_split(rows, cols, 2 * num_sms, most);
+int simt_shares(int rows, int cols, int kp, int num_sms, int most) {
+  // parts: three CTAs per SM
+  const int parts = std::max(1, std::min((3 * num_sms + rows - 1) / std::max(1, rows), most));
+  return simt_split(rows, cols, kp, 2 * num_sms, most, parts);
 }
 
 }  // namespace symnmf

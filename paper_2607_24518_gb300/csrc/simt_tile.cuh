@@ -42,6 +42,7 @@ struct Simt {
   static constexpr int STAGE = S_WORDS + H_WORDS;  // S chunk, H chunk
   static constexpr int WORDS = BUFS * STAGE;
   static constexpr size_t SMEM = sizeof(float) * WORDS;
+  static_assert(NG == (KP <= 16 ? 8 : 128 / KP), "simt_split");
   static_assert(KG % 2 == 0 && 128 * KP <= WORDS && STAGE % 4 == 0, "");
 };
 
@@ -228,11 +229,18 @@ __device__ __forceinline__ void simt_tile(float *sm, const void *S, int64_t lds,
 
 // The number of column shares per row tile that ends soonest: `rows` CTAs per
 // share on `slots` places, each share ceil(cols / s) column tiles long plus
-// about one for its start and end.
-inline int simt_split(int rows, int cols, int slots, int most) {
-  int best = 1;
+// about one for its start and end.  A share's FP32 sums run over 1 / NG of its
+// columns in a row; there are enough shares (of the `most` there may be) that
+// none is longer than with `parts` shares and one group.  Without that limit the
+// rule took a single share for 297 tiles at KP = 64: chains of 19008 FMAs where
+// eight shares had 4864, and an objective off by 2e-8 of the trace, not 6e-10.
+inline int simt_split(int rows, int cols, int kp, int slots, int most, int parts) {
+  const int groups = kp <= 16 ? 8 : 128 / kp;  // Simt<DT, KP>::NG
+  const int64_t longest = (int64_t)groups * ((cols + parts - 1) / parts);
+  int best = 0;
   int64_t cost = INT64_MAX;
   for (int s = 1; s <= most && s <= cols; ++s) {
+    if ((cols + s - 1) / s > longest && s < most) continue;
     const int64_t waves = ((int64_t)rows * s + slots - 1) / slots;
     const int64_t c = waves * ((cols + s - 1) / s + 1);
     if (c < cost) {
@@ -240,7 +248,7 @@ inline int simt_split(int rows, int cols, int slots, int most) {
       best = s;
     }
   }
-  return best;
+  return best > 0 ? best : 1;
 }
 
 }  // namespace symnmf

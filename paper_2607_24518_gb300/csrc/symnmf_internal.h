@@ -168,7 +168,7 @@ constexpr int kSlotStride = 4;
 // launchers (return cudaError_t of the launch)
 cudaError_t launch_prod_simt(const ProdArgs &a, cudaStream_t s);
 // column shares per row tile (ProdArgs::nsplit) of the SIMT product, at most `most`
-int simt_shares(int rows, int cols, int num_sms, int most);
+int simt_shares(int rows, int cols, int kp, int num_sms, int most);
 // tensor-core product; with epi != nullptr (full row and column lists only)
 // the kernel also runs the per-tile epilogue and the cross-tile reduction
 cudaError_t launch_step_tc(const ProdArgs &a, const EpiArgs *epi, int *tile_cnt, cudaStream_t s,

@@ -113,3 +113,21 @@ def test_tile_scalars_of_the_stand_alone_epilogue_are_fp64_sums(L, n, k):
         assert L.symnmf_get_trace(h)[-1].sumA == float(A.astype(np.float64).sum())
     finally:
         L.symnmf_destroy(h)
+
+
+@pytest.mark.parametrize("n,k", [(38000, 64), (38000, 20), (16700, 64), (700, 64)])
+def test_chains_of_the_objective_without_a_handle(L, n, k):
+    """An FP32 chain of m equal terms rounds by at most m / 2 * 2^-24 of its sum
+    (half a unit of a partial sum, whose average is half the sum), and equal
+    terms come near that.  Eight column shares bound a chain by 128 columns of
+    ceil(tiles / 8) tiles, however many shares a call takes; 32 FMAs of the dot
+    with H, 35 of a Gram partial (twice, as its square) and slack add 256."""
+    s, t = 0.640625, np.float32(0.0809360146522522)
+    S = torch.full((n, n), s, dtype=torch.bfloat16, device=DEV)
+    H = torch.full((n, k), float(t), device=DEV)
+    f = torch.zeros(1, dtype=torch.float64, device=DEV)
+    L.symnmf_objective_noalloc(S, n, n, L.BF16, None, 0, H, k, 0.0, f)
+    tr = float(n) * n * k * s * float(t) ** 2
+    g2 = (k * n * float(t) ** 2) ** 2
+    m = 128 * -(-(-(-n // 128)) // 8)
+    assert abs(float(f[0]) - (g2 - 2.0 * tr)) <= (m / 2 + 256) * 2.0 ** -24 * 2.0 * tr
