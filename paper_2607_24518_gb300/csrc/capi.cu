@@ -431,6 +431,10 @@ int prod(symnmf_t h, const int *row_list, int n_rows, const int *col_list, int n
   a.n_rows_list = n_rows;
   a.col_list = col_list;
   a.n_cols_list = n_cols;
+  // (FP32 at kp = 64 forms its products in another way than below, and FP8
+  // pieces of H share a factor per tile: those restarts do not have the bits of
+  // a handle of their own in any case)
+  a.grid_kp = h->dtype == SYMNMF_BF16 ? pad_k(h->k / h->restarts) : h->kp;
   a.batch_tiles = h->batch_tiles;
   a.out = out;
   const int64_t most = std::min<int64_t>(64, h->pq_cap_tiles / std::max(1, n_rows));

@@ -1908,14 +1908,17 @@ cudaError_t launch_step_tc(const ProdArgs &a, const EpiArgs *epi, int *tile_cnt,
   // two grids, so that small ones run side by side (8 handles n <= 8000 k = 16
   // BF16 1826 -> 1630 us for ten iterations, 8 of n <= 4000 k = 32 FP32 1897 ->
   // 1477; one grid in all: 2 of n <= 6000 720 -> 953).
+  // BF16 limits go by the padded rank of one restart (grid_kp), so that restarts
+  // joined in one handle are cut as their separate handles are and add up in
+  // the same order.
   if (epi && a.n_rows_list < num_sms) {
     const int R = a.n_rows_list, cols = a.n_cols_list;
     const int most = std::min(num_sms / R, cols);
-    const int units = a.dtype == 0 ? 4 : a.dtype == 1 ? 12 : a.kp == 64 ? 20 : 14;
+    const int units = a.dtype == 0 ? 4 : a.dtype == 1 ? 12 : a.grid_kp == 64 ? 20 : 14;
     int m = std::min(most, (cols + units - 1) / units);
     if (a.batch_tiles > R) m = std::max(1, std::min(m, 2 * num_sms / a.batch_tiles));
     const int whole = (cols + m - 1) / m, share = (int)((ta.W + ta.G - 1) / ta.G);
-    const int extra = a.dtype == 0 ? (a.kp == 64 ? 0 : 3) : a.dtype == 1 && a.kp == 64 ? 3 : 8;
+    const int extra = a.dtype == 0 ? (a.grid_kp == 64 ? 0 : 3) : a.dtype == 1 && a.grid_kp == 64 ? 3 : 8;
     if (m < most || whole - share <= extra) ta.G = m * R;
   }
   ta.n_cols = a.n_cols_list;

@@ -80,6 +80,7 @@ struct ProdArgs {
   const int *col_list;   // column tile indices (nullptr: all tiles in order)
   int n_cols_list;
   int nsplit;
+  int grid_kp;           // rank that the limits of the grid go by (launch_step_tc)
   int batch_tiles;       // row tiles of all handles stepped together (0: one handle)
   int chain;             // Chain bits: products of one iteration that need nothing of each other
   float *out;

@@ -102,6 +102,38 @@ def test_joint_restarts_bf16_k64(L):
         L.symnmf_destroy(h1)
 
 
+@pytest.mark.parametrize("dtype,n,k,R", [("bf16", 6704, 16, 4), ("bf16", 6704, 32, 2), ("bf16", 1024, 16, 4),
+                                         ("f32", 3000, 8, 4)])
+def test_joint_restarts_equal_separate_handles_bit_for_bit(L, dtype, n, k, R):
+    """On the tensor cores a joint handle takes the grid of one restart's rank,
+    so its blocks add up in the separate handles' order; at n = 6704 a rank-64
+    handle of its own would take another grid.  Bit for bit where both form the
+    products alike: BF16, and FP32 up to joint rank 32 (FP8 pieces of H carry a
+    factor of all columns of a row tile, which joint and separate handles need
+    not share)."""
+    A = np.random.default_rng(n).random((n, 6))
+    S = torch.tensor(np.minimum(1.0, A @ A.T / 3), dtype=torch.float32, device=DEV)
+    H0 = torch.tensor(np.random.default_rng(k).uniform(0.0, 0.1, (n, R * k)), dtype=torch.float32, device=DEV)
+    T = S.to({"f32": torch.float32, "bf16": torch.bfloat16}[dtype])
+    code = {"f32": L.F32, "bf16": L.BF16}[dtype]
+    hp = L.symnmf_hparams_default(L.ADAGRAD, eta=0.1)
+    hj, h1 = L.symnmf_create(T, n, R * k, code), L.symnmf_create(T, n, k, code)
+    try:
+        for h in (hj, h1):
+            assert L.symnmf_get_impl(h) == 2
+        L.symnmf_set_restarts(hj, R)
+        L.symnmf_set_H(hj, H0)
+        L.symnmf_step(hj, hp, 12)
+        Hj = _get(L, hj, n, R * k)
+        for r in (0, R - 1):
+            L.symnmf_set_H(h1, H0[:, r * k:(r + 1) * k].contiguous())
+            L.symnmf_step(h1, hp, 12)
+            assert np.array_equal(Hj[:, r * k:(r + 1) * k], _get(L, h1, n, k)), r
+    finally:
+        L.symnmf_destroy(hj)
+        L.symnmf_destroy(h1)
+
+
 def test_restart_checks_match_separate_records(L):
     """At each check every restart's E_r and KKT measure equal the records
     of its separate solve.  E_r is formed from the gradient the step wrote
