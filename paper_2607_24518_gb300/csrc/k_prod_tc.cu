@@ -123,7 +123,9 @@ struct Cfg {
   static constexpr uint32_t STAGE = A_BYTES + B_BYTES + B2_BYTES;
   // stages per accumulator chain: the tensor core's FP32 accumulation is
   // kept to at most 8 chained MMAs per accumulator, the rest is summed in
-  // FP32 registers
+  // FP32 registers.  (FP32 at kp = 64 chains 12, one stage: eight low-order
+  // products, S H_lo and S_lo H_hi, near 2^-11 of the sum, then the four of full
+  // size that it chained before; gradient errors at tf32_lead)
   static constexpr int FOLD = F32 ? 1 : SPU;
   // accumulator columns per part read before one wait when folding
   static constexpr int FOLD_CW = F32 ? 8 : (KP == 64 ? 16 : 32);
@@ -653,7 +655,7 @@ __device__ __forceinline__ void tile_finish(const EpiArgs &e, int tp, float (&p)
             uint16_t *B16 = bt_b16(e.Btn, KP, e.ldb);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-              const float hi = tf32_trunc(hn[j]);
+              const float hi = tf32_lead<KP>(hn[j]);
               B[(int64_t)(cb + cc + j) * e.ldb + r0 + row] = hi;
               B[(int64_t)(KP + cb + cc + j) * e.ldb + r0 + row] = tf32_round(hn[j] - hi);
               B16[(int64_t)(cb + cc + j) * e.ldb + r0 + row] = bf16_bits(hn[j]);

@@ -7,13 +7,14 @@
 //   * product partial slots are 128 x kp row-major blocks
 //   * the MMA copy of H is stored transposed, [2*kp][ldb] with rows 0..kp-1
 //     = hi(H^T) and kp..2kp-1 = lo(H^T), ldb = ntiles * 128 (columns past n
-//     are 0), in one of two formats (bt_fmt):
-//       0: bfloat16, hi = bf16(H), lo = bf16(H - hi)      (BF16 / FP8 S)
+//     are 0), in one of three formats (bt_fmt):
+//       0: bfloat16, hi = bf16(H), lo = bf16(H - hi)            (BF16 S)
 //       1: float holding tf32 values, hi = H with the 13 low mantissa bits
-//          cleared, lo = (H - hi) rounded to tf32, followed by a bf16
+//          cleared (kp = 64: H rounded to tf32), lo = (H - hi) rounded to
+//          tf32, followed by a bf16
 //          copy [max(kp,16)][ldb] with rows 0..kp-1 = bf16(H^T) and the
 //          rest 0 (the operand of the S_lo H product)      (FP32 S)
-//       2: e4m3 bytes, hi = e4m3(H / d), lo = e4m3(16 (H / d - hi)), with d a
+//       2: e4m3 bytes, hi = e4m3(H / d), lo = e4m3(H / d - hi), with d a
 //          power of two per 128-row tile of H (the smallest with
 //          max|H_tile| / d <= 448); the 2 kp rows are followed by the
 //          ntiles FP32 values d                               (FP8 S)

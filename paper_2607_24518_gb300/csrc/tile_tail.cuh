@@ -91,7 +91,7 @@ __device__ void tile_tail(const float (*Hn)[KP + 1], int64_t r0, void *Bt, int b
     for (int e = tid; e < KP * kTileRows; e += blockDim.x) {
       const int c = e / kTileRows, r = e % kTileRows;
       const float v = Hn[r][c];
-      const float hi = tf32_trunc(v);
+      const float hi = tf32_lead<KP>(v);
       B[(int64_t)c * ldb + r0 + r] = hi;
       B[(int64_t)(KP + c) * ldb + r0 + r] = tf32_round(v - hi);
       B16[(int64_t)c * ldb + r0 + r] = bf16_bits(v);

@@ -151,3 +151,25 @@ def test_tc_free_running_matches_oracle(L, storage):
     # is compared in absolute terms
     assert np.max(np.abs(Eg - Er)) < 5e-6
     assert O.rel_err(Hg, s.H) < 1e-3
+
+
+@pytest.mark.parametrize("n,k", [(256, 33), (256, 64), (132, 50)])
+def test_fp32_rank_64_leaves_out_nothing_of_one_sign(L, n, k):
+    """At kp = 64 the FP32 product leaves S_lo H_lo out.  With S and H one unit
+    below a power of two both truncated pieces would lose 2^-11, and every term
+    2^-22 of its size; H's leading piece is rounded to nearest, so what is left
+    of it is 2^-24.  S_lo rounded to tf32 is off by 2^-24 of S here, the sums of
+    n / 32 equal chains are short and the Gram term, 2^-6 of the other, adds its
+    FP32 error: 2^-23 of the product in all."""
+    S = torch.full((n, n), 1.0 - 2.0 ** -24, device=DEV)
+    H = torch.full((n, k), 2.0 ** -6 * (1.0 - 2.0 ** -24), device=DEV)
+    h = L.symnmf_create(S, n, k, L.F32)
+    try:
+        L.symnmf_set_impl(h, 2)
+        L.symnmf_set_H(h, H)
+        G = _grad(L, h, n, k)
+    finally:
+        L.symnmf_destroy(h)
+    s, x = 1.0 - 2.0 ** -24, 2.0 ** -6 * (1.0 - 2.0 ** -24)
+    ref = 4.0 * (x * (n * k * x * x) - n * s * x)
+    assert np.max(np.abs(np.asarray(G, dtype=np.float64) - ref)) <= 2.0 ** -23 * 4.0 * n * s * x
