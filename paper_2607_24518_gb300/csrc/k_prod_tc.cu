@@ -173,8 +173,7 @@ struct Cfg {
   // 144 us).
   static constexpr bool PTMEM = (KP == 64 && DT == 1);
   static constexpr uint32_t PA0 = PB0 + 2 * KP;
-  static constexpr int NPR = PTMEM ? 0 : KP;  // columns of the sum in registers
-  static constexpr uint32_t TMEM_NEED = PA0 + (uint32_t)(KP - NPR);
+  static constexpr uint32_t TMEM_NEED = PA0 + (PTMEM ? (uint32_t)KP : 0u);
   static constexpr uint32_t TMEM_COLS = TMEM_NEED <= 32 ? 32 : TMEM_NEED <= 64 ? 64 : TMEM_NEED <= 128 ? 128 : TMEM_NEED <= 256 ? 256 : 512;
   static_assert(STAGES >= 2, "shared memory ring too small");
   static_assert(TMEM_NEED <= 512, "tensor memory budget exceeded");
@@ -787,7 +786,7 @@ struct Hand {
   volatile int *sflag;
 };
 
-// Epilogue warps 2-5: one thread per tile row.
+// Epilogue warps 2-9: two threads per tile row, half the columns each.
 template <int DT, int KP>
 __device__ void epilogue_role(const TcArgs &a, const EpiArgs &e, uint32_t tmem_base, float *Hs,
                               double *scratch, const Hand &hd,
@@ -1043,10 +1042,10 @@ __device__ void epilogue_role(const TcArgs &a, const EpiArgs &e, uint32_t tmem_b
   }
 }
 
-// Folder warps 6-9: fold each accumulator chain (<= 16 MMAs) into FP32
-// registers, one thread per tile row, and hand the tile segment's P over.
-// With FP32 storage the same warps first convert each staged S row into
-// its tf32 hi / lo parts in TMEM (the MMA's A operand).
+// Folder warps 10-13: fold each accumulator chain (<= 8 MMAs) into FP32,
+// one thread per tile row, and hand the tile segment's P over.  With FP32
+// storage (kp <= 32) the same warps first convert each staged S row to S_lo
+// in bf16 in TMEM (an MMA's A operand).
 template <int DT, int KP>
 __device__ void folder_role(const TcArgs &a, uint32_t tmem_base, uint8_t *smem, uint64_t *full,
                             uint64_t *empty, uint64_t *afull, uint64_t *aempty, uint64_t *tfull,
@@ -1059,12 +1058,11 @@ __device__ void folder_role(const TcArgs &a, uint32_t tmem_base, uint8_t *smem, 
   const int row = q * 32 + lane;
   const int ft = (warp - 10) * 32 + lane;
   const uint32_t lane_off = (uint32_t)(q * 32) << 16;
-  constexpr int NP = C::NPR;  // columns [0, NP) of the sum in registers, the rest in PA
-  constexpr int NPA = NP > 0 ? NP : 1;
-  float p[NPA];
+  constexpr int NP = C::PTMEM ? 0 : KP;  // columns of the running sum in registers
+  float p[NP > 0 ? NP : 1];
 #pragma unroll
-  for (int c = 0; c < NPA; ++c) p[c] = 0.f;
-  bool pa_first = true;                   // PTMEM: the next fold starts PA (columns [NP, kp))
+  for (int c = 0; c < NP; ++c) p[c] = 0.f;
+  bool pa_first = true;                   // PTMEM: the next fold starts the sum in PA
   const uint32_t tpa = tmem_base + lane_off + C::PA0;
   int acc = 0, pb = 0;
   uint32_t tph = 0u, pph = 0u;  // bit i: parity of accumulator / P buffer i
@@ -1091,17 +1089,16 @@ __device__ void folder_role(const TcArgs &a, uint32_t tmem_base, uint8_t *smem, 
     const uint32_t tb = tmem_base + lane_off + C::PB0 + (uint32_t)(pb * KP);
     if constexpr (C::PTMEM) {
 #pragma unroll
-      for (int cc = NP; cc < KP; cc += 16) {
+      for (int cc = 0; cc < KP; cc += 16) {
         uint32_t x[16];
-        tmem_ld8_nw(tpa + (cc - NP), x, 0);
-        tmem_ld8_nw(tpa + (cc - NP) + 8, x, 8);
+        tmem_ld8_nw(tpa + cc, x, 0);
+        tmem_ld8_nw(tpa + cc + 8, x, 8);
         tmem_wait_ld_all(x);
         tmem_st16(tb + cc, x);
       }
-    }
-    {
+    } else {
 #pragma unroll
-      for (int cc = 0; cc < NP; cc += 8) {
+      for (int cc = 0; cc < KP; cc += 8) {
         float v[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) v[j] = p[cc + j];
@@ -1122,10 +1119,10 @@ __device__ void folder_role(const TcArgs &a, uint32_t tmem_base, uint8_t *smem, 
       float *dst = a.out + ((int64_t)(b + tp) * 128 + row) * KP;
       if constexpr (C::PTMEM) {
 #pragma unroll
-        for (int cc = NP; cc < KP; cc += 16) {
+        for (int cc = 0; cc < KP; cc += 16) {
           uint32_t x[16];
-          tmem_ld8_nw(tpa + (cc - NP), x, 0);
-          tmem_ld8_nw(tpa + (cc - NP) + 8, x, 8);
+          tmem_ld8_nw(tpa + cc, x, 0);
+          tmem_ld8_nw(tpa + cc + 8, x, 8);
           tmem_wait_ld_all(x);
 #pragma unroll
           for (int c4 = 0; c4 < 4; ++c4)
@@ -1142,7 +1139,6 @@ __device__ void folder_role(const TcArgs &a, uint32_t tmem_base, uint8_t *smem, 
     for (int c = 0; c < NP; ++c) p[c] = 0.f;
     pa_first = true;
   };
-  // fold accumulator chain f (stage-sized chunks [f FOLD, (f+1) FOLD))
   // FP8: the scale of each unit (S tile scale over the H tile factor) comes
   // from a shared ring of 2 x 128 entries in this CTA's unit order.  The
   // 128 folder threads load block j + 2 together at the end of block j and
@@ -1198,58 +1194,25 @@ __device__ void folder_role(const TcArgs &a, uint32_t tmem_base, uint8_t *smem, 
     constexpr int NPART = (C::JOIN ? 1 : 2) + (C::NL > 0 ? 1 : 0);
     constexpr int CW = (KP < C::FOLD_CW) ? KP : C::FOLD_CW;
     if constexpr (C::PTMEM) {
-      // columns [0, NP): p += this chain, 16 columns per round
+      // PA = (pa_first ? 0 : PA) + this chain's [H_hi] and [H_lo] parts (BF16)
+      static_assert(!C::PTMEM || (DT == 1 && NPART == 2), "two parts, no scale");
 #pragma unroll
-      for (int cc = 0; cc < NP; cc += 16) {
-        uint32_t x[NPART * 16];
-#pragma unroll
-        for (int u = 0; u < 16; u += 8) {
-          tmem_ld8_nw(tb + cc + u, x, u);
-          if constexpr (!C::JOIN) tmem_ld8_nw(tb + KP + cc + u, x, 16 + u);
-          if constexpr (C::NL > 0) tmem_ld8_nw(tb + C::N + cc + u, x, 32 + u);
-        }
-        tmem_wait_ld_all(x);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          float v;
-          if constexpr (C::JOIN) {
-            v = __uint_as_float(x[j]) * sc;
-          } else if constexpr (C::F8) {
-            v = (__uint_as_float(x[j]) + __uint_as_float(x[16 + j])) * sc;
-          } else {
-            v = __uint_as_float(x[j]) + __uint_as_float(x[16 + j]);
-          }
-          if constexpr (C::NL > 0) v += __uint_as_float(x[32 + j]);
-          p[cc + j] += v;
-        }
-      }
-      // columns [NP, kp): PA = (pa_first ? 0 : PA) + this chain
-#pragma unroll
-      for (int cc = NP; cc < KP; cc += 16) {
-        uint32_t x[(NPART + 1) * 16];
+      for (int cc = 0; cc < KP; cc += 16) {
+        uint32_t x[48];
 #pragma unroll
         for (int u = 0; u < 16; u += 8) {
           tmem_ld8_nw(tb + cc + u, x, u);
-          if constexpr (!C::JOIN) tmem_ld8_nw(tb + KP + cc + u, x, 16 + u);
-          if constexpr (C::NL > 0) tmem_ld8_nw(tb + C::N + cc + u, x, 32 + u);
-          if (!pa_first) tmem_ld8_nw(tpa + (cc - NP) + u, x, NPART * 16 + u);
+          tmem_ld8_nw(tb + KP + cc + u, x, 16 + u);
+          if (!pa_first) tmem_ld8_nw(tpa + cc + u, x, 32 + u);
         }
         tmem_wait_ld_all(x);
         uint32_t o[16];
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-          float v;
-          if constexpr (C::JOIN) {
-            v = __uint_as_float(x[j]) * sc;
-          } else if constexpr (C::F8) {
-            v = (__uint_as_float(x[j]) + __uint_as_float(x[16 + j])) * sc;
-          } else {
-            v = __uint_as_float(x[j]) + __uint_as_float(x[16 + j]);
-          }
-          if constexpr (C::NL > 0) v += __uint_as_float(x[32 + j]);
-          o[j] = __float_as_uint(pa_first ? v : __uint_as_float(x[NPART * 16 + j]) + v);
+          const float v = __uint_as_float(x[j]) + __uint_as_float(x[16 + j]);
+          o[j] = __float_as_uint(pa_first ? v : __uint_as_float(x[32 + j]) + v);
         }
-        tmem_st16(tpa + (cc - NP), o);
+        tmem_st16(tpa + cc, o);
       }
       tmem_wait_st();
       pa_first = false;
