@@ -876,6 +876,10 @@ def run_kmeans(args):
     }
 
 
+# kernels of one build with ||S||^2: preparation, GEMM, sum
+DEP_BUILD_KERNELS = 3
+
+
 def run_dependence(args):
     """The solver's input from data on the GPU (Sec. 3): the absolute
     Pearson correlation of n = 1e5 variables over T = 500 observations of
@@ -974,7 +978,7 @@ def run_dependence(args):
                      "flops_per_launch": piece_flops, "tiles": tiles},
         "cpu_baseline": cpu,
         "clocks": ck,
-        "gpu_launches": 3 * 4,
+        "gpu_launches": 3 * DEP_BUILD_KERNELS,
         "status": "ok",
     }
 

@@ -62,3 +62,10 @@ def test_oracle_row_rate_extrapolates_by_rows():
     r = bench.oracle_row_rate(S, H, np.arange(64), 4096, budget_s=0.2)
     assert r["kind"] == "oracle" and r["value"] > 0
     assert "x 64" in r["sample"]
+
+
+def test_kernels_of_a_dependence_build():
+    """The bench line counts a build's kernels: those its launcher starts."""
+    src = open(os.path.join(bench.ROOT, "paper_2607_24518_gb300", "csrc", "k_dep.cu")).read()
+    launcher = src[src.index("cudaError_t launch_dependence("):]
+    assert bench.DEP_BUILD_KERNELS == launcher.count("<<<")
