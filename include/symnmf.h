@@ -374,7 +374,12 @@ int symnmf_objective_noalloc_check(int64_t n, int64_t lds, int32_t dtype, int32_
  * g_r^2 over its n k/R entries, and only its columns of A are reset (the
  * handle's own controller makes no reset; the record's reset flag says
  * whether any restart reset).  No restart resets at a check where the handle
- * stops.  Call before stepping; the current H's Gram is recomputed.
+ * stops.  A restart of a joint handle agrees with a handle of its own to FP32
+ * rounding; with BF16 storage, and FP32 up to joint rank 32, on the tensor cores
+ * and outside symnmf_batch_step bit for bit (the same grid and order of sums;
+ * FP32 above rank 32 forms its products in another way, FP8 pieces of H share a
+ * factor among the restarts, and the exact-FP32 product adds its column groups in
+ * an order that depends on the rank).  Call before stepping; the current H's Gram is recomputed.
  * Default 1.  The per-restart check state (each restart's E0, previous E
  * and reset state) is not part of the checkpoint blob: after
  * symnmf_set_state it starts again at the next check.

@@ -80,9 +80,11 @@ __device__ void gram_tile(const ObjArgs &a, int tile, float *sm) {
 }
 
 // blockIdx.y < split: a column share; == split: the tile's Gram partial.
-// n = 10000, KP = 32 FP32: 500 -> 188 us (17 TFMA/s of 37); the tile Grams
-// beside the shares and their sum over the chip replace a pass of their own
-// and one CTA's 49 us.
+// n = 10000, KP = 32 FP32: 500 -> 188 us (17 TFMA/s of 37), BF16 695 -> 264, FP8
+// 563 -> 243; KP = 64 527 / 854 / 780 -> 337 / 415 / 397 (128 registers: BF16 and FP8
+// spill 88 to 240 bytes a thread above KP = 8, FP32 68 above KP = 16).  The tile
+// Grams beside the shares and their sum over the chip replace a pass of their
+// own and one CTA's 49 us.
 template <int DT, int KP>
 __global__ void __launch_bounds__(256, 2) tr_share_kernel(ObjArgs a) {
   extern __shared__ __align__(16) float sm_obj[];

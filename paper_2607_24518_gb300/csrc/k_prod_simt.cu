@@ -12,9 +12,14 @@
 namespace symnmf {
 namespace {
 
-// 128 registers for two CTAs per SM.  n = 3001, KP = 16 FP32 33 -> 15 us; n =
-// 5001, KP = 32 BF16 94 -> 57 us (one 16-value block per thread fed by scalar
-// reads, no chunk in flight during the FMAs, before).
+// 128 registers for two CTAs per SM.  BF16 and FP8 above KP = 8 spill 48 to 320
+// bytes a thread under that cap, FP32 above KP = 16 24, and are quicker at every
+// rank all the same than one 16-value block per thread fed by scalar reads with
+// no chunk in flight during the FMAs.  Before -> now in us, KP = 8 / 16 / 32 / 64:
+// n = 3001 FP32 23 / 33 / 45 / 61 -> 11 / 15 / 21 / 35, BF16 22 / 33 / 46 / 68 -> 15 /
+// 19 / 23 / 41, FP8 34 / 33 / 52 / 69 -> 16 / 19 / 24 / 40; n = 10000 FP32 284 / 339 /
+// 442 / 584 -> 80 / 130 / 207 / 367, BF16 216 / 292 / 446 / 761 -> 199 / 209 / 272 /
+// 516, FP8 422 / 287 / 584 / 733 -> 190 / 195 / 268 / 466.
 template <int DT, int KP>
 __global__ void __launch_bounds__(256, 2) prod_simt_kernel(ProdArgs a) {
   extern __shared__ __align__(16) float sm_simt[];

@@ -1,12 +1,14 @@
 """The dependence-matrix builder (Sec. 3) on the GPU against the FP64 oracle.
 
-G = Y^T Y runs on the tensor cores as hi hi + lo hi + hi lo over tf32
-pieces of the FP32 centred values (the dropped lo lo term is below 2^-21
-relative), accumulated in FP32 over K = 3 T' terms; S_ij = |G_ij| /
-sqrt(G_ii G_jj) with FP64 column norms.  Each S_ij is a cosine, so its
-error is bounded by the relative error of G_ij against sqrt(G_ii G_jj):
-2^-21 from the pieces plus the FP32 accumulation, a few units of 2^-24
-times the number of chained MMAs K / 8 in the worst case.  The tests hold
+G = Y^T Y runs on the tensor cores as hi hi + lo hi + hi lo over FP16
+pieces of the FP32 centred values, scaled by a power of two per column (the
+dropped lo lo term is below 2^-24 relative), accumulated in FP32 over K = 3 T'
+terms; S_ij = |G_ij| / sqrt(G_ii G_jj) with column norms of FP64 accuracy.  Each
+S_ij is a cosine, so its error is bounded by the relative error of G_ij against
+sqrt(G_ii G_jj): 2^-22 from the pieces plus the FP32 accumulation, a few units
+of 2^-24 times the number of chained MMAs K / 16 in the worst case
+(test_gpu_dependence_range.py holds that); the bound here is twice as wide, for
+pieces of 11 bits and MMAs of K = 8.  The tests hold
 FP32 output to TOL(T) = 2^-21 + 4 (3 T' / 8) 2^-24, BF16 to that plus half
 a bf16 step (2^-9 for values up to 1), and FP8 codes to the oracle's
 quantiser applied to the oracle's S, allowing one-step differences only
