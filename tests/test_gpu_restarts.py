@@ -102,9 +102,10 @@ def test_joint_restarts_bf16_k64(L):
         L.symnmf_destroy(h1)
 
 
-@pytest.mark.parametrize("dtype,n,k,R", [("bf16", 6704, 16, 4), ("bf16", 6704, 32, 2), ("bf16", 1024, 16, 4),
-                                         ("f32", 3000, 8, 4)])
-def test_joint_restarts_equal_separate_handles_bit_for_bit(L, dtype, n, k, R):
+@pytest.mark.parametrize("dtype,n,k,R,method", [("bf16", 6704, 16, 4, 0), ("bf16", 6704, 32, 2, 0), ("bf16", 1024, 16, 4, 1),
+                                                ("bf16", 1024, 8, 8, 3), ("bf16", 1024, 16, 4, 4), ("bf16", 1024, 32, 2, 5),
+                                                ("f32", 3000, 8, 4, 0), ("f32", 1000, 16, 2, 4), ("f32", 1000, 8, 2, 5)])
+def test_joint_restarts_equal_separate_handles_bit_for_bit(L, dtype, n, k, R, method):
     """On the tensor cores a joint handle takes the grid of one restart's rank,
     so its blocks add up in the separate handles' order; at n = 6704 a rank-64
     handle of its own would take another grid.  Bit for bit where both form the
@@ -116,7 +117,7 @@ def test_joint_restarts_equal_separate_handles_bit_for_bit(L, dtype, n, k, R):
     H0 = torch.tensor(np.random.default_rng(k).uniform(0.0, 0.1, (n, R * k)), dtype=torch.float32, device=DEV)
     T = S.to({"f32": torch.float32, "bf16": torch.bfloat16}[dtype])
     code = {"f32": L.F32, "bf16": L.BF16}[dtype]
-    hp = L.symnmf_hparams_default(L.ADAGRAD, eta=0.1)
+    hp = L.symnmf_hparams_default(method, **(dict(rho=50.0) if method == 5 else dict(eta=0.1)))
     hj, h1 = L.symnmf_create(T, n, R * k, code), L.symnmf_create(T, n, k, code)
     try:
         for h in (hj, h1):
